@@ -81,8 +81,8 @@ typedef enum {
                             (J2D_ERR_ARG otherwise; default 8 and 2); box plans: {4, 6, 8} for
                             FP32, {2, 3, 4} for FP64 (default 8 and 2).  Forward runs of single
                             grids only (adjoint runs and batches take TILES).  AUTO takes it for
-                            FP32 grids too large for the chip and FP64 grids of 8192^2 cells or
-                            more. */
+                            grids too large for the chip (FP64 box plans: of 8192^2 cells or
+                            more). */
 } j2d_algo;
 
 /* Plan options (j2d5pt_set_option / j2d5pt_get_option). */
@@ -309,7 +309,8 @@ j2d_status j2d5pt_arith_info(unsigned *exact_mask, int *exact_guard);
  * stored columns per band (32 vectors' worth minus 2G), bands
  * (ceil(nx / stored columns)), rows stored per run H, runs per band}: band b
  * stores columns [1 + b*(stored), ...) and run r rows [1 + r*H, ...), each
- * clipped to the grid.  J2D_ERR_ARG for sizes < 1, an unknown dtype or shape,
+ * clipped to the grid (FP64 five-point runs too few to fill the device are each
+ * shared by several warps).  J2D_ERR_ARG for sizes < 1, an unknown dtype or shape,
  * a depth with no stream kernel, resident_warps < 1 or a NULL out. */
 j2d_status j2d5pt_stream_geometry(int nx, int ny, j2d_dtype dtype, int shape, int depth, long resident_warps,
                                   long out[6]);

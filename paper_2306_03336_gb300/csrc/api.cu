@@ -895,7 +895,7 @@ extern "C" j2d_status j2d5pt_stream_geometry(int nx, int ny, j2d_dtype dtype, in
   if (resident_warps < 1) return fail(J2D_ERR_ARG, "stream_geometry: resident_warps %ld < 1", resident_warps);
   if (!stream_depth_ok(dtype, depth, shape))
     return fail(J2D_ERR_ARG, "stream_geometry: no stream kernel of depth %d for this dtype and shape", depth);
-  const StreamGeom q = stream_geometry_warps(dtype, nx, ny, depth, resident_warps);
+  const StreamGeom q = stream_geometry_warps(dtype, nx, ny, depth, resident_warps, shape);
   out[0] = q.depth;
   out[1] = q.G;
   out[2] = q.vw;

@@ -22,8 +22,9 @@ template <typename T> struct VecOf;
 template <> struct VecOf<double> { static constexpr int V = 2; using type = double2; };
 template <> struct VecOf<float> { static constexpr int V = 4; using type = float4; };
 
-// The five link weights of one cell: x-1, x+1, y-1, centre, y+1.
-template <typename T> struct Links { T xm, xp, ym, c, yp; };
+// The five link weights of one cell: x-1, x+1, y-1, centre, y+1.  nz is the
+// addend of the chain's first product (see first_product()).
+template <typename T> struct Links { T xm, xp, ym, c, yp, nz = T(-0.0); };
 
 // Base weights as the user gives them: W (x-1), E (x+1), S (y-1), C, N (y+1).
 template <typename T> struct Weights { T w[5]; };
@@ -35,6 +36,23 @@ __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, 
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
+// The FP64 pipe takes an FMA of three vector registers every 64 clocks per
+// warp and SM quarter, but a multiply, an add, or an FMA with a constant-bank
+// or uniform-register operand only every 76 (597 against 502 G/s over the
+// chip at 1.99 GHz, whatever the number of warps).  So FP64 kernels hold
+// their weights in vector registers (vreg(): a shuffle by the lane's own index,
+// which the compiler cannot prove uniform) and take the chain's first product
+// as an FMA that adds -0.0, which rounds exactly as the multiply does, signs
+// of zeros included; the -0.0 is a vector register too (nz), or the compiler
+// would turn the FMA back into a multiply.
+__device__ __forceinline__ double vreg(double v) { return __shfl_sync(0xffffffffu, v, threadIdx.x & 31); }
+__device__ __forceinline__ float vreg(float v) { return v; }  // FP32: no such difference
+template <typename T> __device__ __forceinline__ Links<T> vreg_links(const Links<T> &a) {
+  return {vreg(a.xm), vreg(a.xp), vreg(a.ym), vreg(a.c), vreg(a.yp), vreg(T(-0.0))};
+}
+__device__ __forceinline__ double first_product(double w, double v, double nz) { return fma_rn(w, v, nz); }
+__device__ __forceinline__ float first_product(float w, float v, float) { return mul_rn(w, v); }
+
 // One cell update: the product of the y-1 link, then fused multiply-adds of
 // the centre, x-1, x+1 and y+1 links.  The order starts with the operands a
 // row sweep already holds in registers and ends with the ones that arrive
@@ -42,7 +60,7 @@ __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fm
 // Every kernel uses this one order: results are bit-identical across kernels.
 template <typename T>
 __device__ __forceinline__ T stencil(const Links<T> &a, T xm, T xp, T ym, T c, T yp) {
-  T r = mul_rn(a.ym, ym);
+  T r = first_product(a.ym, ym, a.nz);
   r = fma_rn(a.c, c, r);
   r = fma_rn(a.xm, xm, r);
   r = fma_rn(a.xp, xp, r);
@@ -199,12 +217,19 @@ __device__ __forceinline__ double stencil_cell(const Links<double> &a, const Exa
 // multiply-adds of (y-1, x-1), (y-1, x+1), (y, x), (y, x-1), (y, x+1),
 // (y+1, x), (y+1, x-1), (y+1, x+1): the operands of the row a sweep loads
 // last enter last.  Box9 holds the weights in that chain order.
-template <typename T> struct Box9 { T w[9]; };
+template <typename T> struct Box9 { T w[9], nz = T(-0.0); };
+template <typename T> __device__ __forceinline__ Box9<T> vreg_box(const Box9<T> &b) {
+  Box9<T> r;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) r.w[i] = vreg(b.w[i]);
+  r.nz = vreg(T(-0.0));
+  return r;
+}
 
 // The chain over three rows (m: y-1, c: y, p: y+1), each as (x-1, x, x+1).
 template <typename T>
 __device__ __forceinline__ T stencil_box(const Box9<T> &b, T m0, T m1, T m2, T c0, T c1, T c2, T p0, T p1, T p2) {
-  T r = mul_rn(b.w[0], m1);
+  T r = first_product(b.w[0], m1, b.nz);
   r = fma_rn(b.w[1], m0, r);
   r = fma_rn(b.w[2], m2, r);
   r = fma_rn(b.w[3], c1, r);

@@ -1871,9 +1871,12 @@ DtbConfig dtb_choose(j2d_dtype dt, const std::vector<GridDesc> &grids, int sms, 
     else if (fits && (single || dt == J2D_F64)) algo = J2D_ALGO_RESIDENT;  // FP64 batches: grouped resident
     // grids too large for the chip: the stream schedule for FP32 (16384^2:
     // 4254 GCells/s against 1950 for the best shared-memory schedule; the box
-    // 2578 against 1418) and for large FP64 grids (16384^2: 194 against 162 for
-    // the tiles; 8192^2: 170; at 4096^2 the tiles are faster, 143 against 130)
-    else if (single && !rq.adjoint && (dt == J2D_F32 || (long)grids[0].nx * grids[0].ny >= (8192L << 13)))
+    // 2578 against 1418) and five-point FP64 (16384^2: 259 against 162 for the
+    // tiles; 4096^2: 193 against 145; 2304x1700: 146 against 97; fields of both
+    // signs, which no window takes, 4096^2: 91 against 86), and for large FP64
+    // box grids
+    else if (single && !rq.adjoint &&
+             (dt == J2D_F32 || grids[0].shape == 5 || (long)grids[0].nx * grids[0].ny >= (8192L << 13)))
       algo = J2D_ALGO_STREAM;
     else algo = J2D_ALGO_TILES;
   }

@@ -45,6 +45,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "window.cuh"
 
 namespace j2d {
 
@@ -64,8 +65,8 @@ struct StreamParams {
   int G;        // halo columns on each side of a band (a multiple of V, >= the pass's steps)
   int vw;       // stored (valid) columns per band: 32V - 2G
   int bands;    // column bands
-  int H;        // rows stored per run
-  int runs;     // runs per band
+  int H;        // rows stored per unit
+  int runs;     // units per band
   int meff;     // steps of this pass (<= M: steps t > meff leave rows unchanged)
   void *keep;   // keeping every state: step t's rows go to keep + (t - 1) * keep_stride
   long keep_stride;
@@ -73,6 +74,7 @@ struct StreamParams {
   long nelem;   // elements of each buffer ((ny + 2) * pitch), for the checked build
   int *status;  // checked build: J2D_ERR_BOUNDS is recorded here
   double w[9];  // five-point: W, E, S, C, N; box: the nine weights, rows y-1, y, y+1, columns x-1, x, x+1
+  WindowWeights win;  // FP64 five-point: the weights in windowed fixed point (window.cuh)
 };
 
 // ---- one lane's 16-byte vector of a row, in registers -------------------------
@@ -433,6 +435,207 @@ __device__ __forceinline__ void stream_sweep(const StreamParams &p, const typena
   stage_drain();
 }
 
+// ---- FP64 in windowed fixed point (window.cuh) -----------------------------------
+// The same pipeline with every row also in fixed point: rows y mod 4 in {0, 1} take
+// the exact sum, the others the chain with its first two operations, on the
+// integer pipes.  A sweep picks its window from the first rows it reads and
+// stops before the first row that depends on an interior value outside it; the
+// caller takes the next rows through stream_sweep() and comes back.  Ring values
+// never change, so a sweep does not stop for them: a row beside a ring value
+// outside the window takes its affected cells through the general evaluation.
+struct RowX {
+  double a, b;
+  Fx xa, xb;
+  bool ring_out;  // this lane's ring cell in the row is outside the window
+};
+__device__ __forceinline__ Fx shfl_up_fx(Fx v) {
+  return {__shfl_up_sync(0xffffffffu, v.a0, 1), __shfl_up_sync(0xffffffffu, v.a1, 1)};
+}
+__device__ __forceinline__ Fx shfl_down_fx(Fx v) {
+  return {__shfl_down_sync(0xffffffffu, v.a0, 1), __shfl_down_sync(0xffffffffu, v.a1, 1)};
+}
+
+// A cell of the integer path with a value outside the window, out of line (few
+// cells take it).
+__device__ __noinline__ double general_exact_cell(double W, double E, double S, double C, double N, double xm, double xp,
+                                                  double ym, double c, double yp) {
+  const Links<double> l{W, E, S, C, N};
+  return stencil_cell(l, exact_weights(l), true, xm, xp, ym, c, yp);
+}
+
+// Rows [y0, y1) of the unit; returns the first row not stored (y1: all are), or
+// -1 when the first rows hold a value no window takes.
+template <int M, bool EDGE>
+__device__ __forceinline__ int stream_sweep_window(const StreamParams &p, const Links<double> &lk, long e0, int x0,
+                                                   unsigned hold, bool live, bool st, int y0, int y1, float4 *ring) {
+  constexpr int U = 4, S = 2 * U;
+  const double *in = static_cast<const double *>(p.in);
+  double *out = static_cast<double *>(p.out);
+  const WindowWeights &w = p.win;
+  // trips start on rows congruent to 1 - M mod 4: where a run of whole trips
+  // (y0 = 1 + run * H, H a multiple of 4) needs its first row
+  constexpr int PH = (1 - M) & 3;
+  const int a = y0 - M - ((y0 - M - PH) & 3);
+  const int iend = y1 + M;
+  const bool short_pass = p.meff < M;
+  const uint32_t base = smem_u32(ring);
+#pragma unroll
+  for (int j = 0; j < kAhead; ++j) issue_row(in, p, a + j, e0, live && a + j >= 0, base + 512u * j);
+  // columns of this lane outside the logical array hold a value of the window
+  const bool oa = EDGE && (x0 < 0 || x0 > p.nx + 1), ob = EDGE && (x0 + 1 < 0 || x0 + 1 > p.nx + 1);
+  if (EDGE) hold |= (oa ? 1u : 0u) | (ob ? 2u : 0u);
+  // window: its top one binade above the largest interior value of the first rows
+  stage_drain();
+  int top = 0, low = 0x7fffffff;  // high words: negative for negative values
+#pragma unroll
+  for (int j = 0; j < kAhead; ++j) {
+    const double2 v = *reinterpret_cast<const double2 *>(ring + 32 * j);
+    if (a + j < 1 || a + j > p.ny) continue;
+    if (!EDGE || !(hold & 1u)) top = max(top, __double2hiint(v.x)), low = min(low, __double2hiint(v.x));
+    if (!EDGE || !(hold & 2u)) top = max(top, __double2hiint(v.y)), low = min(low, __double2hiint(v.y));
+  }
+  Window q;
+  if (!window_set(q, w, __reduce_max_sync(0xffffffffu, top) >> 20) || __any_sync(0xffffffffu, low < 0x100000)) return -1;
+  const double dummy = window_dummy(q);
+  RowX A[M], B[M];
+  {
+    uint32_t d = 0;
+    const Fx x = window_conv(dummy, q, d);
+#pragma unroll
+    for (int t = 0; t < M; ++t) A[t] = B[t] = RowX{dummy, dummy, x, x, false};
+  }
+  // a row's fixed-point form; d collects the distances of its interior values
+  // (none in the ring rows and beyond)
+  auto conv = [&](RowX &r, bool ring_row, uint32_t &d) {
+    uint32_t da = 0, db = 0;
+    r.xa = window_conv(r.a, q, da);
+    r.xb = window_conv(r.b, q, db);
+    if (EDGE) {
+      r.ring_out = ((hold & 1u) && da >= w.lim) || ((hold & 2u) && db >= w.lim);
+      if (hold & 1u) da = 0;
+      if (hold & 2u) db = 0;
+    }
+    if (!ring_row) d |= da | db;
+  };
+  // the asynchronous copies' source (row i + kAhead) and the stored row's
+  // address, advanced a row per iteration
+  const long step = live ? p.pitch : 0;
+  const double *src = in + (live ? (long)(a + kAhead) * p.pitch + e0 : 0);
+  double *dst = out + ((long)(a - M) * p.pitch + e0);
+  // Iteration i: row i of step 0 arrives (ph = i mod 4); false: some interior
+  // value is outside the window.  chk: a trip with rows that are not stored, near
+  // the ring rows or past the grid, or a pass of fewer than M steps.
+  auto iter = [&](int i, const float4 *slot, uint32_t fill, int ph, bool chk) -> bool {
+    stage_wait();
+    const double2 v = *reinterpret_cast<const double2 *>(slot);
+    {
+      bool on = live && (!chk || i + kAhead <= p.ny + 1);
+      if (on) on = stream_ok(src - in, 2, p);
+      stage_copy(fill, chk || kChecked ? (on ? src : in) : src, on);
+      src += step;
+    }
+    RowX cur{v.x, v.y, {}, {}, false};
+    if (EDGE && oa) cur.a = dummy;
+    if (EDGE && ob) cur.b = dummy;
+    if (chk && i > p.ny + 1) cur.a = cur.b = dummy;
+    uint32_t d = 0;
+    conv(cur, chk && (i < 1 || i > p.ny), d);
+#pragma unroll
+    for (int t = 1; t <= M; ++t) {
+      const RowX &c = B[t - 1], &ym = A[t - 1];
+      const int r = i - t;
+      RowX n;
+      n.ring_out = false;
+      // a row beside the ring rows, or beside a ring column's value outside the window
+      const bool beside = (chk && (r == 1 || r == p.ny)) || (EDGE && __any_sync(0xffffffffu, c.ring_out));
+      if (((ph - t + 4 * M) & 3) < 2) {
+        const Fx L = shfl_up_fx(c.xb), R = shfl_down_fx(c.xa);
+        n.a = window_exact(w, q, L, c.xb, ym.xa, c.xa, cur.xa);
+        n.b = window_exact(w, q, c.xa, R, ym.xb, c.xb, cur.xb);
+        if ((EDGE || chk) && beside) {
+          const double l = __shfl_up_sync(0xffffffffu, c.b, 1), rr = __shfl_down_sync(0xffffffffu, c.a, 1);
+          uint32_t da = 0, db = 0;
+          for (double u : {l, c.b, ym.a, c.a, cur.a}) window_conv(u, q, da);
+          for (double u : {c.a, rr, ym.b, c.b, cur.b}) window_conv(u, q, db);
+          if (da >= w.lim) n.a = general_exact_cell(p.w[0], p.w[1], p.w[2], p.w[3], p.w[4], l, c.b, ym.a, c.a, cur.a);
+          if (db >= w.lim) n.b = general_exact_cell(p.w[0], p.w[1], p.w[2], p.w[3], p.w[4], c.a, rr, ym.b, c.b, cur.b);
+          __syncwarp();
+        }
+      } else {
+        const double L = __shfl_up_sync(0xffffffffu, c.b, 1), R = __shfl_down_sync(0xffffffffu, c.a, 1);
+        if ((EDGE || chk) && beside) {
+          n.a = stencil(lk, L, c.b, ym.a, c.a, cur.a);
+          n.b = stencil(lk, c.a, R, ym.b, c.b, cur.b);
+        } else {
+          n.a = window_head<2>(w, q, {2, 3}, {ym.xa, c.xa});
+          n.b = window_head<2>(w, q, {2, 3}, {ym.xb, c.xb});
+          n.a = fma_rn(lk.yp, cur.a, fma_rn(lk.xp, c.b, fma_rn(lk.xm, L, n.a)));
+          n.b = fma_rn(lk.yp, cur.b, fma_rn(lk.xp, R, fma_rn(lk.xm, c.a, n.b)));
+        }
+      }
+      if (EDGE && (hold & 1u)) n.a = c.a;
+      if (EDGE && (hold & 2u)) n.b = c.b;
+      if (chk && (r == 0 || r == p.ny + 1 || t > p.meff)) {
+        n.a = c.a;
+        n.b = c.b;
+      }
+      if (t < M) conv(n, chk && (r < 1 || r > p.ny), d);
+      A[t - 1] = B[t - 1];
+      B[t - 1] = cur;
+      cur = n;
+    }
+    if (__any_sync(0xffffffffu, d >= w.lim)) return false;
+    const int r = i - M;
+    if (st && (!chk || (r >= y0 && r < y1)) && stream_ok(dst - out, 2, p)) row_store(dst, RowD{cur.a, cur.b});
+    dst += p.pitch;
+    return true;
+  };
+  int s = 0;
+  auto trip = [&](int i, bool chk) -> int {  // U iterations; U, or the one that found a value outside the window
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int sn = s + u + kAhead;
+      if (!iter(i + u, ring + 32 * (s + u), base + 512u * (sn >= S ? sn - S : sn), (u + PH) & 3, chk)) return u;
+    }
+    s = s == 0 ? U : 0;
+    return U;
+  };
+  // steady trips: every row stored, all copied rows inside the grid
+  const int lo = max(y0 + M, M + 2), hi = short_pass ? 0 : min(y1 + M, p.ny + 2 - kAhead) - U;  // [lo, hi]: first rows
+  for (int i = a; i < iend; i += U) {
+    const int n = EDGE || i < lo || i > hi ? trip(i, true) : trip(i, false);
+    if (n != U) {
+      stage_drain();
+      return max(y0, i + n - M);
+    }
+  }
+  stage_drain();
+  return y1;
+}
+
+// A unit in windowed fixed point where its values allow it; elsewhere stretches
+// of rows by the general sweep: eight rows, four times as many while the window
+// keeps failing soon after, and all of them where a value is not positive.
+template <int M, bool EDGE>
+__device__ __forceinline__ void stream_unit_window(const StreamParams &p, const WeightsD &k, long e0, int x0,
+                                                   unsigned hold, bool live, bool st, int y0, int y1, float4 *ring) {
+  int stretch = p.win.lim ? 8 : y1;
+  while (y0 < y1) {
+    if (p.win.lim) {
+      const int y = stream_sweep_window<M, EDGE>(p, k.l, e0, x0, hold, live, st, y0, y1, ring);
+      if (y < 0) stretch = y1;
+      else if (y - y0 >= 16) stretch = 8;
+      y0 = max(y, y0);
+    }
+    if (y0 < y1) {
+      const int ye = y0 + min(stretch, y1 - y0);
+      stream_sweep<double, M, EDGE, true, false, 5>(p, k, e0, x0, hold, live, st, y0, ye, ring);
+      y0 = ye;
+      stretch = min(4 * stretch, 1 << 20);
+    }
+  }
+}
+
 __device__ __forceinline__ void make_weights(const StreamParams &p, WeightsF *k) {
   const float w = (float)p.w[0], e = (float)p.w[1], s = (float)p.w[2], c = (float)p.w[3], n = (float)p.w[4];
   k->w = make_float2(w, w);
@@ -447,16 +650,24 @@ __device__ __forceinline__ void make_weights(const StreamParams &p, WeightsF9 *k
   for (int i = 0; i < 9; ++i) k->w[i] = make_float2(b.w[i], b.w[i]);
 }
 __device__ __forceinline__ void make_weights(const StreamParams &p, WeightsD9 *k) {
-  k->b = box_chain<double>(p.w);
-  k->u = box_exact_weights(k->b);
+  k->b = vreg_box(box_chain<double>(p.w));
+  k->u = box_exact_weights(box_chain<double>(p.w));
 }
 __device__ __forceinline__ void make_weights(const StreamParams &p, WeightsD *k) {
-  k->l = Links<double>{p.w[0], p.w[1], p.w[2], p.w[3], p.w[4]};
-  k->u = exact_weights(k->l);
+  const Links<double> l{p.w[0], p.w[1], p.w[2], p.w[3], p.w[4]};
+  k->l = vreg_links(l);
+  k->u = exact_weights(l);
 }
 
+// Kernels whose units run in windowed fixed point.  Registers: at M = 2 five
+// blocks of four warps (96 a thread, a few spilled in the rare branches) measured
+// faster than four or six (FP64 16384^2: 259, 252 and 255 GCells/s).
 template <typename T, int M, bool IP, bool KEEP, int SH>
-__global__ void __launch_bounds__(32 * WarpsOf<T>::W) stream_kernel(StreamParams p) {
+constexpr bool kWindowed = std::is_same<T, double>::value && M <= 4 && IP && !KEEP && SH == 5;
+
+template <typename T, int M, bool IP, bool KEEP, int SH>
+__global__ void __launch_bounds__(32 * WarpsOf<T>::W, kWindowed<T, M, IP, KEEP, SH> ? 7 - M : 0)
+    stream_kernel(StreamParams p) {
   constexpr int V = VecOf<T>::V;
   const int lane = threadIdx.x & 31;
   const int unit = blockIdx.x * WarpsOf<T>::W + (threadIdx.x >> 5);
@@ -480,7 +691,12 @@ __global__ void __launch_bounds__(32 * WarpsOf<T>::W) stream_kernel(StreamParams
   make_weights(p, &k);
   __shared__ float4 ring[WarpsOf<T>::W][2 * TripOf<T>::U * 32];
   float4 *mine = &ring[threadIdx.x >> 5][lane];
-  if (edge)
+  if constexpr (kWindowed<T, M, IP, KEEP, SH>) {
+    if (edge)
+      stream_unit_window<M, true>(p, k, e0, x0, hold, live, st, y0, y1, mine);
+    else
+      stream_unit_window<M, false>(p, k, e0, x0, hold, live, st, y0, y1, mine);
+  } else if (edge)
     stream_sweep<T, M, true, IP, KEEP, SH>(p, k, e0, x0, hold, live, st, y0, y1, mine);
   else
     stream_sweep<T, M, false, IP, KEEP, SH>(p, k, e0, x0, hold, live, st, y0, y1, mine);
@@ -548,10 +764,10 @@ static int stream_occupancy(j2d_dtype dt, int m, int shape) {
 StreamGeom stream_geometry(j2d_dtype dt, const GridDesc &g, int depth, int sms) {
   const int d = std::max(1, std::min(depth, stream_max_depth(dt)));
   const long warps = (long)stream_occupancy(dt, d, g.shape) * stream_warps(dt) * std::max(sms, 1);
-  return stream_geometry_warps(dt, g.nx, g.ny, depth, warps);
+  return stream_geometry_warps(dt, g.nx, g.ny, depth, warps, g.shape);
 }
 
-StreamGeom stream_geometry_warps(j2d_dtype dt, int nx, int ny, int depth, long warps) {
+StreamGeom stream_geometry_warps(j2d_dtype dt, int nx, int ny, int depth, long warps, int shape) {
   StreamGeom q;
   const int V = dt == J2D_F64 ? 2 : 4;
   q.depth = std::max(1, std::min(depth, stream_max_depth(dt)));
@@ -559,18 +775,31 @@ StreamGeom stream_geometry_warps(j2d_dtype dt, int nx, int ny, int depth, long w
   q.vw = 32 * V - 2 * q.G;
   q.bands = (nx + q.vw - 1) / q.vw;
   // Several waves of units per pass, so that the block scheduler balances
-  // the SMs as units finish (FP64 k = 2 on 16384^2: 159 GCells/s with one
-  // wave of units, 178 / 191 / 194 / 189 / 175 with 2 / 4 / 8 / 16 / 32;
-  // FP32 k = 8: 3958, 4254 with 2 or 3, 4235 with 4, 4090 with 8), each run
-  // at least 32M (FP64) or 16M (FP32) rows tall, its 2M-row overlap then
-  // costing at most 6% or 12% (FP64 8192^2: 169.7 GCells/s against 164.8 with
-  // 16M; FP32 4096^2: 2764 against 2175 with 32M).
+  // the SMs as units finish, each run at least 32M (FP64) or 16M (FP32) rows tall,
+  // its 2M-row overlap then costing at most 6% or 12% (FP32 k = 8, 16384^2: 3958
+  // GCells/s with one wave, 4254 with 2 or 3, 4235 with 4, 4090 with 8; FP32
+  // 4096^2: 2764 against 2175 with 32M).
   warps = std::max(warps, 1L);
-  const int waves = dt == J2D_F64 ? 8 : 3;
   const int hmin = (dt == J2D_F64 ? 32 : 16) * q.depth;
-  int runs = (int)std::max<long>(1, waves * warps / q.bands);
-  runs = std::min(runs, std::max(1, ny / hmin));
-  q.H = (ny + runs - 1) / runs;
+  if (dt == J2D_F64 && shape == 5) {
+    // Whole waves of units, up to eight with runs of at least 44M rows (k = 2,
+    // 8192^2: 212, 233, 236, 238, 239 and 235 GCells/s with 1, 2, 3, 4, 6 and 8
+    // waves, 16384^2: 258 with 6, 259 with 8, 258 with 16); one wave for
+    // smaller grids (4096^2: 193 with one, 185 with one and a half, 187 with
+    // three).  A run has a whole number of the sweep's four-row trips.
+    const long r1 = std::max<long>(1, warps / q.bands);
+    const long waves = std::min<long>(8, std::max<long>(1, ny / (r1 * 44 * q.depth)));
+    const long hu = ((ny + waves * r1 - 1) / (waves * r1) + 3) / 4 * 4;
+    q.H = (int)std::min<long>(ny, std::max<long>(hu, hmin));
+    // too few units of that height for one wave: the warps share the runs
+    q.hu = (int)std::min<long>(q.H, std::max<long>(hu, 8));
+  } else {
+    const int waves = dt == J2D_F64 ? 8 : 3;
+    int runs = (int)std::max<long>(1, waves * warps / q.bands);
+    runs = std::min(runs, std::max(1, ny / hmin));
+    q.H = (ny + runs - 1) / runs;
+    q.hu = q.H;
+  }
   q.runs = (ny + q.H - 1) / q.H;
   return q;
 }
@@ -590,8 +819,8 @@ cudaError_t launch_stream_pass(j2d_dtype dt, const void *in, void *out, const Gr
   p.G = q.G;
   p.vw = q.vw;
   p.bands = q.bands;
-  p.H = q.H;
-  p.runs = q.runs;
+  p.H = q.hu;
+  p.runs = (g.ny + q.hu - 1) / q.hu;
   p.meff = m;
   p.keep = keep;
   p.keep_stride = keep_stride;
@@ -599,9 +828,11 @@ cudaError_t launch_stream_pass(j2d_dtype dt, const void *in, void *out, const Gr
   p.nelem = (long)(g.ny + 2) * g.pitch;
   p.status = status;
   for (int i = 0; i < 9; ++i) p.w[i] = g.w[i];
+  p.win = WindowWeights{};
+  if (dt == J2D_F64 && g.shape == 5) p.win = window_weights({g.w[0], g.w[1], g.w[2], g.w[3], g.w[4]});
   StreamFn fn = stream_fn(dt, q.depth, ipath, keep != nullptr, g.shape);
   if (!fn || m < 1 || m > q.depth) return cudaErrorInvalidValue;
-  const long units = (long)q.bands * q.runs;
+  const long units = (long)q.bands * p.runs;
   const int W = stream_warps(dt);
   const unsigned blocks = (unsigned)((units + W - 1) / W);
   fn<<<blocks, 32 * W, 0, s>>>(p);

@@ -1,0 +1,85 @@
+"""FP64 stream sweeps in windowed fixed point against the one-step kernel, bit
+for bit: values at and beyond the window's two ends (inside the grid, in the
+ring rows and columns, at the edges of runs), fields no window holds, fields whose
+window moves down the rows, weights at the limits of the fixed-point form (the
+widest spread it takes, one more, a zero, a negative, significands of all ones)."""
+import numpy as np
+import pytest
+
+from paper_2306_03336_gb300 import j2d5pt, synth
+
+pytestmark = pytest.mark.gpu
+
+ONES = float(np.nextafter(1.0, 0.0))
+WEIGHTS = {
+    "equal": [0.2] * 5,
+    "spread4": [0.5, 0.25, 0.04, 0.15, 0.06],
+    "spread5": [0.55, 0.2, 0.0175, 0.13, 0.1],
+    "spread7": [0.55, 0.2, 0.0043, 0.13, 0.11],
+    "spread8": [0.55, 0.2, 0.0021, 0.13, 0.11],
+    "spread9": [0.55, 0.2, 0.0011, 0.13, 0.11],
+    "all_large": [0.24, 0.24, 0.24, 0.24, 0.0012],
+    "all_ones": [ONES / 4, ONES / 8, ONES / 4, ONES / 4, ONES / 8],
+    "zero": [0.25, 0.25, 0.0, 0.25, 0.25],
+    "negative": [0.3, 0.3, -0.1, 0.25, 0.25],
+    "large": [30.0, 20.0, 10.0, 25.0, 15.0],
+}
+
+
+def field(name, nx, ny):
+    r = np.random.default_rng(5)
+    u = 0.5 + 0.5 * r.random((ny + 2, nx + 2))
+    if name == "uniform":
+        return r.random((ny + 2, nx + 2))
+    if name == "spikes":  # single cells at both ends of the window and beyond it
+        for v in [2.0 ** -6, 2.0 ** -7, 2.0 ** -7 * ONES, 2.0 ** -8, 1.0, 2.0, 2.0 * ONES, 4.0, 0.0, -1.0, 5e-324]:
+            u[r.integers(0, ny + 2), r.integers(0, nx + 2)] = v
+    elif name == "ring":  # ring values outside the window
+        for edge in (u[0], u[-1], u[:, 0], u[:, -1]):
+            edge[:] = r.choice([0.0, 1e-3, 0.7, 1e3, -2.0], size=edge.shape)
+    elif name == "zero_ring":
+        u[0], u[-1], u[:, 0], u[:, -1] = 0.0, 0.0, 0.0, 0.0
+    elif name == "ramp":  # a window of its own every few rows
+        u *= 2.0 ** (np.arange(ny + 2)[:, None] // 7 % 40 - 20)
+    elif name == "wide":
+        u *= 2.0 ** r.integers(-40, 40, size=u.shape)
+    elif name == "tiny":  # below every window
+        u *= 2.0 ** -1019
+    elif name == "huge":
+        u *= 2.0 ** 1000
+    elif name == "short":  # rounding ties
+        u = np.floor(u * 2 ** 12) / 2 ** 12
+    return u
+
+
+def run(u, w, nx, ny, steps, algo, depth):
+    plan = j2d5pt.Plan(nx, ny, "f64", w).set("algo", algo).set("depth", depth)
+    src, dst = plan.to_device(u), plan.empty()
+    plan.run(src, dst, steps)
+    plan.sync()
+    got = plan.to_host(dst)
+    plan.close()
+    return got
+
+
+@pytest.mark.parametrize("fname", ["uniform", "spikes", "ring", "zero_ring", "ramp", "wide", "tiny", "huge", "short"])
+@pytest.mark.parametrize("nx,ny", [(1, 1), (3, 2), (61, 70), (124, 129), (187, 301)])
+def test_window_fields(fname, nx, ny):
+    u = field(fname, nx, ny)
+    w = np.array(WEIGHTS["spread4"])
+    for depth, steps in ((2, 5), (3, 7), (4, 8)):
+        ref = run(u, w, nx, ny, steps, "onestep", 0)
+        got = run(u, w, nx, ny, steps, "stream", depth)
+        assert np.array_equal(got, ref), "k=%d: %d cells differ" % (depth, np.count_nonzero(got != ref))
+
+
+@pytest.mark.parametrize("wname", sorted(WEIGHTS))
+def test_window_weights(wname):
+    nx, ny = 130, 203
+    w = np.array(WEIGHTS[wname])
+    for fname in ("spikes", "short"):
+        u = field(fname, nx, ny)
+        for depth, steps in ((2, 4), (3, 3)):
+            ref = run(u, w, nx, ny, steps, "onestep", 0)
+            got = run(u, w, nx, ny, steps, "stream", depth)
+            assert np.array_equal(got, ref), "%s k=%d: %d cells differ" % (fname, depth, np.count_nonzero(got != ref))
