@@ -78,11 +78,11 @@ typedef enum {
                             rows, advancing k steps per pass as a pipeline held in registers
                             (step t of row i-t as row i arrives); one launch per pass, no shared
                             memory.  k in {4, 6, 8, 10, 12} for FP32, {2, 3, 4, 6} for FP64
-                            (J2D_ERR_ARG otherwise; default 8 and 2); box plans: {4, 6, 8} for
-                            FP32, {2, 3, 4} for FP64 (default 8 and 2).  Forward runs of single
+                            (J2D_ERR_ARG otherwise; default 8, or 6 below 3200^2 cells, and 2);
+                            box plans: {4, 6, 8} for FP32, {2, 3, 4} for FP64 (default 6 and 2).  Forward runs of single
                             grids only (adjoint runs and batches take TILES).  AUTO takes it for
-                            grids too large for the chip (FP64 box plans: of 8192^2 cells or
-                            more). */
+                            FP32 grids and for FP64 grids too large for the chip (FP64 box
+                            plans: of 8192^2 cells or more). */
 } j2d_algo;
 
 /* Plan options (j2d5pt_set_option / j2d5pt_get_option). */
@@ -133,8 +133,8 @@ j2d_status j2d5pt_plan_batched(j2d5pt_plan_t *plan, int count, const int *nx, co
  * j2d5pt_run / j2d5pt_run_host / j2d5pt_autotune and the option, layout,
  * describe, timing and status calls; its algorithms are J2D_ALGO_ONESTEP,
  * J2D_ALGO_SKEWED and J2D_ALGO_STREAM (any other choice runs the skewed
- * tiles; AUTO takes the stream schedule for FP32 grids too large for the
- * chip and FP64 grids of 8192^2 cells or more).  The adjoint,
+ * tiles; AUTO takes the stream schedule for FP32 grids and FP64 grids of
+ * 8192^2 cells or more).  The adjoint,
  * weight-gradient and j2d5pt_set_weights calls return J2D_ERR_UNSUPPORTED.
  * FP64 cells are evaluated as j2d5pt_arith_info describes, with the nine
  * terms: the FMA chain takes the product of the (y-1, x) term, then the
@@ -309,8 +309,8 @@ j2d_status j2d5pt_arith_info(unsigned *exact_mask, int *exact_guard);
  * stored columns per band (32 vectors' worth minus 2G), bands
  * (ceil(nx / stored columns)), rows stored per run H, runs per band}: band b
  * stores columns [1 + b*(stored), ...) and run r rows [1 + r*H, ...), each
- * clipped to the grid (FP64 five-point runs too few to fill the device are each
- * shared by several warps).  J2D_ERR_ARG for sizes < 1, an unknown dtype or shape,
+ * clipped to the grid (runs too few to fill the device are each shared by
+ * several warps).  J2D_ERR_ARG for sizes < 1, an unknown dtype or shape,
  * a depth with no stream kernel, resident_warps < 1 or a NULL out. */
 j2d_status j2d5pt_stream_geometry(int nx, int ny, j2d_dtype dtype, int shape, int depth, long resident_warps,
                                   long out[6]);

@@ -217,19 +217,12 @@ __device__ __forceinline__ double stencil_cell(const Links<double> &a, const Exa
 // multiply-adds of (y-1, x-1), (y-1, x+1), (y, x), (y, x-1), (y, x+1),
 // (y+1, x), (y+1, x-1), (y+1, x+1): the operands of the row a sweep loads
 // last enter last.  Box9 holds the weights in that chain order.
-template <typename T> struct Box9 { T w[9], nz = T(-0.0); };
-template <typename T> __device__ __forceinline__ Box9<T> vreg_box(const Box9<T> &b) {
-  Box9<T> r;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) r.w[i] = vreg(b.w[i]);
-  r.nz = vreg(T(-0.0));
-  return r;
-}
+template <typename T> struct Box9 { T w[9]; };
 
 // The chain over three rows (m: y-1, c: y, p: y+1), each as (x-1, x, x+1).
 template <typename T>
 __device__ __forceinline__ T stencil_box(const Box9<T> &b, T m0, T m1, T m2, T c0, T c1, T c2, T p0, T p1, T p2) {
-  T r = first_product(b.w[0], m1, b.nz);
+  T r = mul_rn(b.w[0], m1);
   r = fma_rn(b.w[1], m0, r);
   r = fma_rn(b.w[2], m2, r);
   r = fma_rn(b.w[3], c1, r);
@@ -350,6 +343,11 @@ template <> __device__ __forceinline__ float lds_s<float>(uint32_t a) {
   asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
   return v;
 }
+
+// Programmatic dependent launch: let the next kernel of the stream start; wait
+// until the kernels before this one have finished and their writes are visible.
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // mbarrier (shared memory transaction barrier) for TMA completion.
 __device__ __forceinline__ void mbar_init(uint64_t *bar, int count) {

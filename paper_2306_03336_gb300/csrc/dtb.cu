@@ -1868,7 +1868,11 @@ DtbConfig dtb_choose(j2d_dtype dt, const std::vector<GridDesc> &grids, int sms, 
                            : !rq.adjoint && groups_fit(grids, sw, c.ctas, c.rows);
   if (algo == J2D_ALGO_AUTO) {
     if (rq.steps < 4) algo = J2D_ALGO_ONESTEP;
-    else if (fits && (single || dt == J2D_F64)) algo = J2D_ALGO_RESIDENT;  // FP64 batches: grouped resident
+    // FP64 grids that fit on chip (batches: grouped resident); FP32 keeps them
+    // there only in the adjoint, the stream schedule advancing them faster at every
+    // size (2048x1536: 1.9 against 3.3 us a step, 1024^2: 1.8 against 2.7, 512^2: 1.4
+    // against 2.0)
+    else if (fits && (dt == J2D_F64 || (single && rq.adjoint))) algo = J2D_ALGO_RESIDENT;
     // grids too large for the chip: the stream schedule for FP32 (16384^2:
     // 4254 GCells/s against 1950 for the best shared-memory schedule; the box
     // 2578 against 1418) and five-point FP64 (16384^2: 259 against 162 for the
@@ -1896,7 +1900,11 @@ DtbConfig dtb_choose(j2d_dtype dt, const std::vector<GridDesc> &grids, int sms, 
     c.sweep = 2;
     c.rows = dtb_rows_max_pair(dt, smem_optin);
   }
-  if (algo == J2D_ALGO_STREAM && rq.depth <= 0) c.depth = dt == J2D_F64 ? 2 : 8;
+  // FP32: eight steps a pass for large five-point grids (16384^2: 4660 GCells/s, 4260
+  // with six), six for smaller ones, whose units are short (2048x1536: 2.3 against
+  // 1.9 us a step), and for the box (16384^2: 2445 against 2744)
+  if (algo == J2D_ALGO_STREAM && rq.depth <= 0)
+    c.depth = dt == J2D_F64 ? 2 : (long)grids[0].nx * grids[0].ny >= (3200L * 3200) && grids[0].shape == 5 ? 8 : 6;
   if (algo == J2D_ALGO_SKEWED) {
     c.rows = dtb_rows_max_skew(dt, smem_optin);
     if (rq.depth <= 0) c.depth = dt == J2D_F64 ? 8 : 16;

@@ -293,6 +293,7 @@ template <typename T, int M, bool EDGE, bool IP, bool KEEP, int SH> struct Pipe 
   unsigned hold;  // ring columns in this lane's vector
   bool st;        // this lane's vector is stored
   int y0, y1;     // stored rows [y0, y1)
+  T *dst;         // FP32: this lane's vector of the row an iteration finishes (set by the sweep, advanced a row each time)
 
   __device__ __forceinline__ Pipe(const W &k_, const StreamParams &p_, T *out_, long e0_, int x0_, unsigned hold_,
                                   bool st_, int y0_, int y1_)
@@ -305,8 +306,9 @@ template <typename T, int M, bool EDGE, bool IP, bool KEEP, int SH> struct Pipe 
   }
 
   // Iteration i: row i of step 0 arrives; steps 1..M advance one row each.
-  // CHK: some step reaches ring row 0 or ny + 1 in this iteration, or the
-  // pass has fewer than M steps (steps beyond meff pass their rows through).
+  // CHK: some step reaches ring row 0 or ny + 1 in this iteration, the row it
+  // finishes may not be one to store, or the pass has fewer than M steps (steps
+  // beyond meff pass their rows through).
   // ph: i mod 4 when the caller knows it at compile time (FP64 trips), so
   // that each step's integer-path choice (exact_cell(): rows y mod 4 in
   // {0, 1}) is a constant; -1 otherwise.
@@ -328,9 +330,14 @@ template <typename T, int M, bool EDGE, bool IP, bool KEEP, int SH> struct Pipe 
       }
     }
     const int r = i - M;
-    if (!KEEP && st && r >= y0 && r < y1) {
-      const long e = (long)r * p.pitch + e0;
-      if (stream_ok(e, VecOf<T>::V, p)) row_store(out + e, cur);
+    if constexpr (sizeof(T) == 8) {
+      if (!KEEP && st && r >= y0 && r < y1) {
+        const long e = (long)r * p.pitch + e0;
+        if (stream_ok(e, VecOf<T>::V, p)) row_store(out + e, cur);
+      }
+    } else if (!KEEP) {
+      if (st && (!CHK || (r >= y0 && r < y1)) && stream_ok(dst - out, VecOf<T>::V, p)) row_store(dst, cur);
+      dst += p.pitch;
     }
   }
 };
@@ -410,27 +417,68 @@ __device__ __forceinline__ void stream_sweep(const StreamParams &p, const typena
 #pragma unroll
   for (int j = 0; j < kAhead; ++j) issue_row(in, p, a + j, e0, live, base + 512u * j);
   int s = 0;  // slot of row i: 0 or U
-  for (int i = a; i < iend; i += U) {
-    if (short_pass || i <= M || i + U - 1 >= p.ny + 2) {
+  if constexpr (sizeof(T) == 8) {
+    // FP64: addresses from the row number (running ones cost registers these
+    // kernels do not have: box k = 2, 16384^2, 92 -> 86 GCells/s)
+    for (int i = a; i < iend; i += U) {
+      if (short_pass || i <= M || i + U - 1 >= p.ny + 2) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        stage_wait();
-        const R c = read_slot(ring + 32 * (s + u), (R *)nullptr);
-        const int sn = s + u + kAhead;
-        issue_row(in, p, i + u + kAhead, e0, live, base + 512u * (sn >= S ? sn - S : sn));
-        pipe.template iter<true>(i + u, c, U == 4 ? u : -1);
-      }
-    } else {
+        for (int u = 0; u < U; ++u) {
+          stage_wait();
+          const R c = read_slot(ring + 32 * (s + u), (R *)nullptr);
+          const int sn = s + u + kAhead;
+          issue_row(in, p, i + u + kAhead, e0, live, base + 512u * (sn >= S ? sn - S : sn));
+          pipe.template iter<true>(i + u, c, u);
+        }
+      } else {
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        stage_wait();
-        const R c = read_slot(ring + 32 * (s + u), (R *)nullptr);
-        const int sn = s + u + kAhead;
-        issue_row(in, p, i + u + kAhead, e0, live, base + 512u * (sn >= S ? sn - S : sn));
-        pipe.template iter<false>(i + u, c, U == 4 ? u : -1);
+        for (int u = 0; u < U; ++u) {
+          stage_wait();
+          const R c = read_slot(ring + 32 * (s + u), (R *)nullptr);
+          const int sn = s + u + kAhead;
+          issue_row(in, p, i + u + kAhead, e0, live, base + 512u * (sn >= S ? sn - S : sn));
+          pipe.template iter<false>(i + u, c, u);
+        }
       }
+      s = s == 0 ? U : 0;
     }
-    s = s == 0 ? U : 0;
+  } else {
+    // FP32: the copies' source (row i + kAhead) and the stored row's address
+    // advance a row per iteration, and steady trips (every finished row stored, all
+    // copied rows inside the grid, no step at a ring row) test nothing; a run's
+    // first and last trips and short passes do (k = 8, 16384^2: 4260 -> 4670
+    // GCells/s, of an issue-bound sweep)
+    const long step = live ? p.pitch : 0;
+    const T *src = in + (live ? (long)(a + kAhead) * p.pitch + e0 : 0);
+    pipe.dst = out + ((long)(a - M) * p.pitch + e0);
+    const int lo = max(y0 + M, M + 1), hi = short_pass ? -1 : min(y1 + M, p.ny + 2 - kAhead) - U;
+    for (int i = a; i < iend; i += U) {
+      if (i < lo || i > hi) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          stage_wait();
+          const R c = read_slot(ring + 32 * (s + u), (R *)nullptr);
+          const int sn = s + u + kAhead;
+          bool on = live && i + u + kAhead <= p.ny + 1;
+          if (on) on = stream_ok(src - in, VecOf<T>::V, p);
+          stage_copy(base + 512u * (sn >= S ? sn - S : sn), on ? src : in, on);
+          src += step;
+          pipe.template iter<true>(i + u, c, -1);
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          stage_wait();
+          const R c = read_slot(ring + 32 * (s + u), (R *)nullptr);
+          const int sn = s + u + kAhead;
+          const bool on = kChecked ? live && stream_ok(src - in, VecOf<T>::V, p) : live;
+          stage_copy(base + 512u * (sn >= S ? sn - S : sn), kChecked && !on ? in : src, on);
+          src += step;
+          pipe.template iter<false>(i + u, c, -1);
+        }
+      }
+      s = s == 0 ? U : 0;
+    }
   }
   stage_drain();
 }
@@ -448,20 +496,6 @@ struct RowX {
   Fx xa, xb;
   bool ring_out;  // this lane's ring cell in the row is outside the window
 };
-__device__ __forceinline__ Fx shfl_up_fx(Fx v) {
-  return {__shfl_up_sync(0xffffffffu, v.a0, 1), __shfl_up_sync(0xffffffffu, v.a1, 1)};
-}
-__device__ __forceinline__ Fx shfl_down_fx(Fx v) {
-  return {__shfl_down_sync(0xffffffffu, v.a0, 1), __shfl_down_sync(0xffffffffu, v.a1, 1)};
-}
-
-// A cell of the integer path with a value outside the window, out of line (few
-// cells take it).
-__device__ __noinline__ double general_exact_cell(double W, double E, double S, double C, double N, double xm, double xp,
-                                                  double ym, double c, double yp) {
-  const Links<double> l{W, E, S, C, N};
-  return stencil_cell(l, exact_weights(l), true, xm, xp, ym, c, yp);
-}
 
 // Rows [y0, y1) of the unit; returns the first row not stored (y1: all are), or
 // -1 when the first rows hold a value no window takes.
@@ -650,8 +684,8 @@ __device__ __forceinline__ void make_weights(const StreamParams &p, WeightsF9 *k
   for (int i = 0; i < 9; ++i) k->w[i] = make_float2(b.w[i], b.w[i]);
 }
 __device__ __forceinline__ void make_weights(const StreamParams &p, WeightsD9 *k) {
-  k->b = vreg_box(box_chain<double>(p.w));
-  k->u = box_exact_weights(box_chain<double>(p.w));
+  k->b = box_chain<double>(p.w);
+  k->u = box_exact_weights(k->b);
 }
 __device__ __forceinline__ void make_weights(const StreamParams &p, WeightsD *k) {
   const Links<double> l{p.w[0], p.w[1], p.w[2], p.w[3], p.w[4]};
@@ -659,14 +693,26 @@ __device__ __forceinline__ void make_weights(const StreamParams &p, WeightsD *k)
   k->u = exact_weights(l);
 }
 
-// Kernels whose units run in windowed fixed point.  Registers: at M = 2 five
-// blocks of four warps (96 a thread, a few spilled in the rare branches) measured
-// faster than four or six (FP64 16384^2: 259, 252 and 255 GCells/s).
+// Kernels whose units run in windowed fixed point.
 template <typename T, int M, bool IP, bool KEEP, int SH>
 constexpr bool kWindowed = std::is_same<T, double>::value && M <= 4 && IP && !KEEP && SH == 5;
 
+// Resident blocks per SM asked of the compiler (0: its own choice).  Windowed, M = 2:
+// five blocks of four warps (96 registers, some spilled in the rare branches)
+// measured faster than four or six (FP64 16384^2: 259, 252 and 255 GCells/s).
+// Deep FP32 pipelines and the FP64 box: the occupancy they have had without
+// steady-trip registers on top (FP32 k = 12, 16384^2: 4126 GCells/s at 12 warps,
+// 3872 at 10).
+template <typename T, int M, bool IP, bool KEEP, int SH> constexpr int stream_blocks() {
+  if (kWindowed<T, M, IP, KEEP, SH>) return 7 - M;
+  if (KEEP) return 0;
+  if (std::is_same<T, float>::value && SH == 5) return M == 10 ? 13 : M == 12 ? 12 : 0;
+  if (std::is_same<T, float>::value) return M == 8 ? 12 : 0;
+  return 0;
+}
+
 template <typename T, int M, bool IP, bool KEEP, int SH>
-__global__ void __launch_bounds__(32 * WarpsOf<T>::W, kWindowed<T, M, IP, KEEP, SH> ? 7 - M : 0)
+__global__ void __launch_bounds__(32 * WarpsOf<T>::W, stream_blocks<T, M, IP, KEEP, SH>())
     stream_kernel(StreamParams p) {
   constexpr int V = VecOf<T>::V;
   const int lane = threadIdx.x & 31;
@@ -691,6 +737,7 @@ __global__ void __launch_bounds__(32 * WarpsOf<T>::W, kWindowed<T, M, IP, KEEP, 
   make_weights(p, &k);
   __shared__ float4 ring[WarpsOf<T>::W][2 * TripOf<T>::U * 32];
   float4 *mine = &ring[threadIdx.x >> 5][lane];
+  grid_dependency_wait();  // the pass before this one has finished and its rows are visible
   if constexpr (kWindowed<T, M, IP, KEEP, SH>) {
     if (edge)
       stream_unit_window<M, true>(p, k, e0, x0, hold, live, st, y0, y1, mine);
@@ -700,6 +747,7 @@ __global__ void __launch_bounds__(32 * WarpsOf<T>::W, kWindowed<T, M, IP, KEEP, 
     stream_sweep<T, M, true, IP, KEEP, SH>(p, k, e0, x0, hold, live, st, y0, y1, mine);
   else
     stream_sweep<T, M, false, IP, KEEP, SH>(p, k, e0, x0, hold, live, st, y0, y1, mine);
+  grid_launch_dependents();  // this warp's rows are written: the next pass may be launched (it waits above for them)
 }
 
 // ---- host side ------------------------------------------------------------------
@@ -798,7 +846,12 @@ StreamGeom stream_geometry_warps(j2d_dtype dt, int nx, int ny, int depth, long w
     int runs = (int)std::max<long>(1, waves * warps / q.bands);
     runs = std::min(runs, std::max(1, ny / hmin));
     q.H = (ny + runs - 1) / runs;
-    q.hu = q.H;
+    // smaller grids: one wave of shorter units, at least 3.5M rows (FP32 2048x1536,
+    // k = 6: 2.4, 2.1 and 2.8 us a step with a quarter, half and one wave of
+    // units, before passes overlapped; 3.3 on chip; 3000^2: 3.8 and 3.5 with half
+    // and one)
+    const long r1 = std::max<long>(1, warps / q.bands);
+    q.hu = (int)std::min<long>(q.H, std::max<long>((ny + r1 - 1) / r1, 7 * q.depth / 2));
   }
   q.runs = (ny + q.H - 1) / q.H;
   return q;
@@ -835,9 +888,21 @@ cudaError_t launch_stream_pass(j2d_dtype dt, const void *in, void *out, const Gr
   const long units = (long)q.bands * p.runs;
   const int W = stream_warps(dt);
   const unsigned blocks = (unsigned)((units + W - 1) / W);
-  fn<<<blocks, 32 * W, 0, s>>>(p);
+  // Programmatic dependent launch: the next pass is launched when every warp of
+  // this one has stored its rows, and waits in the kernel for the end of this
+  // one (FP32, 1024^2, k = 6: 1.74 -> 1.45 us a step; released at a kernel's
+  // start instead, its waiting blocks take slots from the running pass: 1.87).
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(32 * W);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
   note_launch();
-  return cudaGetLastError();
+  return cudaLaunchKernelEx(&cfg, fn, p);
 }
 
 }  // namespace j2d

@@ -77,6 +77,13 @@ struct Fx {
   uint32_t a0, a1;
 };
 
+__device__ __forceinline__ Fx shfl_up_fx(Fx v) {
+  return {__shfl_up_sync(0xffffffffu, v.a0, 1), __shfl_up_sync(0xffffffffu, v.a1, 1)};
+}
+__device__ __forceinline__ Fx shfl_down_fx(Fx v) {
+  return {__shfl_down_sync(0xffffffffu, v.a0, 1), __shfl_down_sync(0xffffffffu, v.a1, 1)};
+}
+
 // The window of a warp: cref = eref << 20, cb = (eref + emin - 1035) << 20.
 struct Window {
   uint32_t cref, cb;
@@ -141,6 +148,14 @@ __device__ __forceinline__ double window_exact(const WindowWeights &w, const Win
   uint32_t hi, lo;
   const uint32_t p = window_round(S0, S1, S2, hi, lo);
   return window_compose(p, hi, lo, q);
+}
+
+// A cell of the integer path with a value outside the window, out of line (few
+// cells take it).
+static __device__ __noinline__ double general_exact_cell(double W, double E, double S, double C, double N, double xm,
+                                                         double xp, double ym, double c, double yp) {
+  const Links<double> l{W, E, S, C, N};
+  return stencil_cell(l, exact_weights(l), true, xm, xp, ym, c, yp);
 }
 
 // The first NI operations of the FMA chain, RN(.. RN(W[t1] x1 + RN(W[t0] x0))), each
