@@ -623,11 +623,12 @@ extern "C" j2d_status j2d5pt_run_states(j2d5pt_plan_t p, const void *in, void *s
   p->ran = true;
   cudaError_t e;
   if ((e = launch_ring_copy(p->dtype, in, states, g, s, steps, se)) != cudaSuccess) return cuda_fail(e, "run_states: rings");
-  // AUTO keeps the states with the one-step kernel, which writes every state
-  // anyway: FP64 4096^2, 49 states, 6.48 ms against 6.81 for tiles storing
-  // each step (the stores cost the tiled sweep 18%)
+  // AUTO keeps the states of FP64 grids too large for the chip with the stream
+  // passes (4096^2: 101 us a state against 132 for the one-step kernel; fields of
+  // both signs, which no window takes, 181 against 171), of others with the one-step
+  // kernel, which writes every state anyway
   DtbConfig c = resolve(p, steps, false);
-  if (p->opt_algo == J2D_ALGO_AUTO) c.algo = J2D_ALGO_ONESTEP;
+  if (p->opt_algo == J2D_ALGO_AUTO && !(c.algo == J2D_ALGO_STREAM && p->dtype == J2D_F64)) c.algo = J2D_ALGO_ONESTEP;
   if (c.algo == J2D_ALGO_ONESTEP) {
     const void *src = in;
     for (long t = 0; t < steps; ++t) {

@@ -1882,6 +1882,10 @@ DtbConfig dtb_choose(j2d_dtype dt, const std::vector<GridDesc> &grids, int sms, 
     else if (single && !rq.adjoint &&
              (dt == J2D_F32 || grids[0].shape == 5 || (long)grids[0].nx * grids[0].ny >= (8192L << 13)))
       algo = J2D_ALGO_STREAM;
+    // FP64 adjoint runs of larger grids: the one-step kernel (4096^2: 98 us a step
+    // against 134 for the tiles, 2304x1700: 28 against 49; fields of both signs 163
+    // against 198 and 46 against 66)
+    else if (single && rq.adjoint && dt == J2D_F64) algo = J2D_ALGO_ONESTEP;
     else algo = J2D_ALGO_TILES;
   }
   if (algo == J2D_ALGO_RESIDENT && !fits) algo = single ? J2D_ALGO_BANDS : J2D_ALGO_TILES;

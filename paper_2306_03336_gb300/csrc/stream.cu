@@ -499,7 +499,7 @@ struct RowX {
 
 // Rows [y0, y1) of the unit; returns the first row not stored (y1: all are), or
 // -1 when the first rows hold a value no window takes.
-template <int M, bool EDGE>
+template <int M, bool EDGE, bool KEEP>
 __device__ __forceinline__ int stream_sweep_window(const StreamParams &p, const Links<double> &lk, long e0, int x0,
                                                    unsigned hold, bool live, bool st, int y0, int y1, float4 *ring) {
   constexpr int U = 4, S = 2 * U;
@@ -620,7 +620,18 @@ __device__ __forceinline__ int stream_sweep_window(const StreamParams &p, const 
     }
     if (__any_sync(0xffffffffu, d >= w.lim)) return false;
     const int r = i - M;
-    if (st && (!chk || (r >= y0 && r < y1)) && stream_ok(dst - out, 2, p)) row_store(dst, RowD{cur.a, cur.b});
+    if (KEEP) {
+      // every step's finished row (B[t] holds step t's until the next iteration)
+#pragma unroll
+      for (int t = 1; t <= M; ++t) {
+        const RowX &n = t < M ? B[t < M ? t : 0] : cur;
+        if (st && t <= p.meff && i - t >= y0 && i - t < y1 && stream_ok(dst - out + (M - t) * p.pitch, 2, p))
+          row_store(static_cast<double *>(p.keep) + (t - 1) * p.keep_stride + (dst - out) + (M - t) * p.pitch,
+                    RowD{n.a, n.b});
+      }
+    } else if (st && (!chk || (r >= y0 && r < y1)) && stream_ok(dst - out, 2, p)) {
+      row_store(dst, RowD{cur.a, cur.b});
+    }
     dst += p.pitch;
     return true;
   };
@@ -650,20 +661,20 @@ __device__ __forceinline__ int stream_sweep_window(const StreamParams &p, const 
 // A unit in windowed fixed point where its values allow it; elsewhere stretches
 // of rows by the general sweep: eight rows, four times as many while the window
 // keeps failing soon after, and all of them where a value is not positive.
-template <int M, bool EDGE>
+template <int M, bool EDGE, bool KEEP>
 __device__ __forceinline__ void stream_unit_window(const StreamParams &p, const WeightsD &k, long e0, int x0,
                                                    unsigned hold, bool live, bool st, int y0, int y1, float4 *ring) {
   int stretch = p.win.lim ? 8 : y1;
   while (y0 < y1) {
     if (p.win.lim) {
-      const int y = stream_sweep_window<M, EDGE>(p, k.l, e0, x0, hold, live, st, y0, y1, ring);
+      const int y = stream_sweep_window<M, EDGE, KEEP>(p, k.l, e0, x0, hold, live, st, y0, y1, ring);
       if (y < 0) stretch = y1;
       else if (y - y0 >= 16) stretch = 8;
       y0 = max(y, y0);
     }
     if (y0 < y1) {
       const int ye = y0 + min(stretch, y1 - y0);
-      stream_sweep<double, M, EDGE, true, false, 5>(p, k, e0, x0, hold, live, st, y0, ye, ring);
+      stream_sweep<double, M, EDGE, true, KEEP, 5>(p, k, e0, x0, hold, live, st, y0, ye, ring);
       y0 = ye;
       stretch = min(4 * stretch, 1 << 20);
     }
@@ -695,7 +706,7 @@ __device__ __forceinline__ void make_weights(const StreamParams &p, WeightsD *k)
 
 // Kernels whose units run in windowed fixed point.
 template <typename T, int M, bool IP, bool KEEP, int SH>
-constexpr bool kWindowed = std::is_same<T, double>::value && M <= 4 && IP && !KEEP && SH == 5;
+constexpr bool kWindowed = std::is_same<T, double>::value && M <= 4 && IP && SH == 5;
 
 // Resident blocks per SM asked of the compiler (0: its own choice).  Windowed, M = 2:
 // five blocks of four warps (96 registers, some spilled in the rare branches)
@@ -740,9 +751,9 @@ __global__ void __launch_bounds__(32 * WarpsOf<T>::W, stream_blocks<T, M, IP, KE
   grid_dependency_wait();  // the pass before this one has finished and its rows are visible
   if constexpr (kWindowed<T, M, IP, KEEP, SH>) {
     if (edge)
-      stream_unit_window<M, true>(p, k, e0, x0, hold, live, st, y0, y1, mine);
+      stream_unit_window<M, true, KEEP>(p, k, e0, x0, hold, live, st, y0, y1, mine);
     else
-      stream_unit_window<M, false>(p, k, e0, x0, hold, live, st, y0, y1, mine);
+      stream_unit_window<M, false, KEEP>(p, k, e0, x0, hold, live, st, y0, y1, mine);
   } else if (edge)
     stream_sweep<T, M, true, IP, KEEP, SH>(p, k, e0, x0, hold, live, st, y0, y1, mine);
   else

@@ -83,3 +83,54 @@ def test_window_weights(wname):
             ref = run(u, w, nx, ny, steps, "onestep", 0)
             got = run(u, w, nx, ny, steps, "stream", depth)
             assert np.array_equal(got, ref), "%s k=%d: %d cells differ" % (fname, depth, np.count_nonzero(got != ref))
+
+
+@pytest.mark.parametrize("fname", ["uniform", "spikes", "ramp", "wide", "tiny", "short"])
+@pytest.mark.parametrize("nx,ny", [(130, 12), (131, 9), (323, 70)])
+def test_window_adjoint_items(fname, nx, ny):
+    """Windowed items of the one-step adjoint, alone and with the weight gradient
+    fused, against the tiles (no window)."""
+    import torch
+    for wname in ("spread4", "spread5", "spread9"):
+        lam = field(fname, nx, ny)
+        plan = j2d5pt.Plan(nx, ny, "f64", np.array(WEIGHTS[wname]))
+        src, got, ref = plan.to_device(lam), plan.empty(), plan.empty()
+        for steps in (1, 4):
+            plan.set("algo", "tiles").set("depth", 2).run_adjoint(src, ref, steps)
+            plan.set("algo", "onestep").run_adjoint(src, got, steps)
+            plan.sync()
+            assert np.array_equal(plan.to_host(got), plan.to_host(ref)), (wname, steps)
+        u = plan.to_device(synth.field(nx, ny, 31))
+        dw, dw2 = (torch.zeros(5, dtype=torch.float64, device="cuda") for _ in range(2))
+        plan.set("algo", "tiles").run_adjoint(src, ref, 1)
+        plan.adjoint_step_wgrad(u, src, got, dw)
+        plan.weight_grad(u, src, dw2)
+        plan.sync()
+        assert np.array_equal(plan.to_host(got), plan.to_host(ref)), wname
+        # two fixed summation orders of the same nx * ny products
+        a, b = dw.cpu().numpy(), dw2.cpu().numpy()
+        bound = 2.0 ** -52 * nx * ny * np.abs(lam).max() * 1.0
+        assert np.all(np.abs(a - b) <= bound * nx * ny), wname
+        plan.close()
+
+
+@pytest.mark.parametrize("fname", ["uniform", "spikes", "ring", "ramp", "short"])
+def test_window_states(fname):
+    """State-keeping stream runs: every state against chained one-step runs."""
+    nx, ny, steps = 187, 301, 7
+    u = field(fname, nx, ny)
+    for depth in (2, 3, 4):
+        plan = j2d5pt.Plan(nx, ny, "f64", np.array(WEIGHTS["spread4"]))
+        src = plan.to_device(u)
+        states = plan.empty_states(steps)
+        plan.set("algo", "stream").set("depth", depth).run_states(src, states, steps)
+        plan.sync()
+        plan.set("algo", "onestep")
+        cur = src
+        for t in range(steps):
+            nxt = plan.empty()
+            plan.run(cur, nxt, 1)
+            plan.sync()
+            assert np.array_equal(plan.to_host(states[t]), plan.to_host(nxt)), (depth, t)
+            cur = nxt
+        plan.close()
