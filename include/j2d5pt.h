@@ -81,8 +81,9 @@ typedef enum {
                             (J2D_ERR_ARG otherwise; default 8, or 6 below 3200^2 cells, and 2);
                             box plans: {4, 6, 8} for FP32, {2, 3, 4} for FP64 (default 6 and 2).  Forward runs of single
                             grids only (adjoint runs and batches take TILES).  AUTO takes it for
-                            FP32 grids and for FP64 grids too large for the chip (FP64 box
-                            plans: of 8192^2 cells or more). */
+                            FP32 grids, for FP64 grids too large for the chip and for FP64
+                            box grids (weights within about 32 times of each other, or
+                            8192^2 cells or more). */
 } j2d_algo;
 
 /* Plan options (j2d5pt_set_option / j2d5pt_get_option). */
@@ -133,8 +134,9 @@ j2d_status j2d5pt_plan_batched(j2d5pt_plan_t *plan, int count, const int *nx, co
  * j2d5pt_run / j2d5pt_run_host / j2d5pt_autotune and the option, layout,
  * describe, timing and status calls; its algorithms are J2D_ALGO_ONESTEP,
  * J2D_ALGO_SKEWED and J2D_ALGO_STREAM (any other choice runs the skewed
- * tiles; AUTO takes the stream schedule for FP32 grids and FP64 grids of
- * 8192^2 cells or more).  The adjoint,
+ * tiles; AUTO takes the stream schedule for FP32 grids and, when the weights
+ * lie within about 32 times of each other or the grid has 8192^2 cells or
+ * more, for FP64 grids).  The adjoint,
  * weight-gradient and j2d5pt_set_weights calls return J2D_ERR_UNSUPPORTED.
  * FP64 cells are evaluated as j2d5pt_arith_info describes, with the nine
  * terms: the FMA chain takes the product of the (y-1, x) term, then the

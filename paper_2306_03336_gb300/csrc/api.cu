@@ -14,6 +14,7 @@
 #include "common.cuh"
 #include "dtb.h"
 #include "internal.h"
+#include "window.cuh"
 
 using namespace j2d;
 
@@ -293,6 +294,8 @@ static DtbConfig resolve(j2d5pt_plan_t p, long steps, bool adj) {
   rq.steps = steps;
   rq.adjoint = adj;
   rq.sweep_steps = p->opt_sweep_steps;
+  const GridDesc &g = p->grids[0];
+  rq.windowed = int_path_of(p) && g.shape == 9 && window_weights(box_chain<double>(g.w).w).lim != 0;
   return dtb_choose(p->dtype, p->grids, p->sms, p->smem_optin, rq);
 }
 
@@ -896,7 +899,7 @@ extern "C" j2d_status j2d5pt_stream_geometry(int nx, int ny, j2d_dtype dtype, in
   if (resident_warps < 1) return fail(J2D_ERR_ARG, "stream_geometry: resident_warps %ld < 1", resident_warps);
   if (!stream_depth_ok(dtype, depth, shape))
     return fail(J2D_ERR_ARG, "stream_geometry: no stream kernel of depth %d for this dtype and shape", depth);
-  const StreamGeom q = stream_geometry_warps(dtype, nx, ny, depth, resident_warps, shape);
+  const StreamGeom q = stream_geometry_warps(dtype, nx, ny, depth, resident_warps);
   out[0] = q.depth;
   out[1] = q.G;
   out[2] = q.vw;

@@ -18,6 +18,7 @@ struct DtbRequest {
   long steps = 0;
   bool adjoint = false;
   int sweep_steps = 2;  // TILES, FP32 forward: steps per sweep (J2D_OPT_SWEEP_STEPS)
+  bool windowed = false;  // FP64 box: the plan's weights fit windowed fixed point (window.cuh) and the integer path is on
 };
 
 // Everything one temporally blocked run needs.

@@ -74,7 +74,8 @@ struct StreamParams {
   long nelem;   // elements of each buffer ((ny + 2) * pitch), for the checked build
   int *status;  // checked build: J2D_ERR_BOUNDS is recorded here
   double w[9];  // five-point: W, E, S, C, N; box: the nine weights, rows y-1, y, y+1, columns x-1, x, x+1
-  WindowWeights win;  // FP64 five-point: the weights in windowed fixed point (window.cuh)
+  WindowWeights win;       // FP64: the weights in windowed fixed point (window.cuh), five-point
+  WindowWeightsN<9> win9;  // and box
 };
 
 // ---- one lane's 16-byte vector of a row, in registers -------------------------
@@ -236,6 +237,16 @@ __device__ __forceinline__ RowF9 row_step9(const WeightsF9 &k, const RowF9 &ym, 
 }
 __device__ __forceinline__ RowD9 row_step9(const WeightsD9 &k, const RowD9 &ym, const RowD9 &c, const RowD9 &yp,
                                            bool ea, bool eb) {
+  // the integer path wants nine positive normal values: in a field of both signs
+  // few of a row's 64 cells have them, and a row without any skips the attempt
+  // (300 instructions a cell)
+  if (ea || eb) {
+    const int lo = min(min(__double2hiint(ym.a), __double2hiint(ym.b)),
+                       min(min(__double2hiint(c.a), __double2hiint(c.b)), min(__double2hiint(yp.a), __double2hiint(yp.b))));
+    const int la = min(lo, min(__double2hiint(ym.L), min(__double2hiint(c.L), __double2hiint(yp.L))));
+    const int lb = min(lo, min(__double2hiint(ym.R), min(__double2hiint(c.R), __double2hiint(yp.R))));
+    if (!__any_sync(0xffffffffu, max(la, lb) >= 0x100000)) ea = eb = false;
+  }
   return {stencil_box_cell(k.b, k.u, ea, ym.L, ym.a, ym.b, c.L, c.a, c.b, yp.L, yp.a, yp.b),
           stencil_box_cell(k.b, k.u, eb, ym.a, ym.b, ym.R, c.a, c.b, c.R, yp.a, yp.b, yp.R), 0.0, 0.0};
 }
@@ -371,7 +382,7 @@ __device__ __forceinline__ void stage_drain() { asm volatile("cp.async.wait_all;
 // past the ring row ny + 1, and vectors outside the row, read as zero).
 template <typename T>
 __device__ __forceinline__ void issue_row(const T *in, const StreamParams &p, int i, long e0, bool live, uint32_t dst) {
-  bool on = live && i <= p.ny + 1;
+  bool on = live && i >= 0 && i <= p.ny + 1;
   const long e = on ? (long)i * p.pitch + e0 : 0;
   if (on) on = stream_ok(e, VecOf<T>::V, p);
   stage_copy(dst, in + (on ? e : 0), on);
@@ -408,8 +419,12 @@ __device__ __forceinline__ void stream_sweep(const StreamParams &p, const typena
   const T *in = static_cast<const T *>(p.in);
   T *out = static_cast<T *>(p.out);
   Pipe<T, M, EDGE, IP, KEEP, SH> pipe(k, p, out, e0, x0, hold, st, y0, y1);
-  int a = max(y0 - M, 0);  // earlier rows only warm the pipeline up
-  if (U == 4) a &= ~3;
+  // the first row the last stored row's pipeline needs; FP64 trips start on rows
+  // congruent to PH mod 4, where a unit of whole trips (y0 = 1 + a multiple of 4)
+  // needs its first
+  constexpr int PH = (1 - M) & 3;
+  int a = max(y0 - M, 0);
+  if (U == 4) a = y0 - M - ((y0 - M - PH) & 3);
   const int iend = y1 + M;  // the last iteration stores row y1 - 1
   const bool short_pass = p.meff < M;
   // this lane's slot j is ring[32 * j]; row a + n sits in slot n mod S
@@ -428,7 +443,7 @@ __device__ __forceinline__ void stream_sweep(const StreamParams &p, const typena
           const R c = read_slot(ring + 32 * (s + u), (R *)nullptr);
           const int sn = s + u + kAhead;
           issue_row(in, p, i + u + kAhead, e0, live, base + 512u * (sn >= S ? sn - S : sn));
-          pipe.template iter<true>(i + u, c, u);
+          pipe.template iter<true>(i + u, c, (u + PH) & 3);
         }
       } else {
 #pragma unroll
@@ -437,7 +452,7 @@ __device__ __forceinline__ void stream_sweep(const StreamParams &p, const typena
           const R c = read_slot(ring + 32 * (s + u), (R *)nullptr);
           const int sn = s + u + kAhead;
           issue_row(in, p, i + u + kAhead, e0, live, base + 512u * (sn >= S ? sn - S : sn));
-          pipe.template iter<false>(i + u, c, u);
+          pipe.template iter<false>(i + u, c, (u + PH) & 3);
         }
       }
       s = s == 0 ? U : 0;
@@ -497,15 +512,28 @@ struct RowX {
   bool ring_out;  // this lane's ring cell in the row is outside the window
 };
 
+// The chain's weights and the window of a shape.
+template <int SH> struct WindowCoef {
+  using L = Links<double>;
+  static __device__ __forceinline__ const WindowWeights &window(const StreamParams &p) { return p.win; }
+};
+template <> struct WindowCoef<9> {
+  using L = Box9<double>;
+  static __device__ __forceinline__ const WindowWeightsN<9> &window(const StreamParams &p) { return p.win9; }
+};
+// Operations of the box's nine-term chain on the integer pipes: the y - 1 row's, so
+// that its doubles are not needed again.
+constexpr int kBoxHead = 3;
+
 // Rows [y0, y1) of the unit; returns the first row not stored (y1: all are), or
 // -1 when the first rows hold a value no window takes.
-template <int M, bool EDGE, bool KEEP>
-__device__ __forceinline__ int stream_sweep_window(const StreamParams &p, const Links<double> &lk, long e0, int x0,
+template <int M, bool EDGE, bool KEEP, int SH>
+__device__ __forceinline__ int stream_sweep_window(const StreamParams &p, const typename WindowCoef<SH>::L &lk, long e0, int x0,
                                                    unsigned hold, bool live, bool st, int y0, int y1, float4 *ring) {
   constexpr int U = 4, S = 2 * U;
   const double *in = static_cast<const double *>(p.in);
   double *out = static_cast<double *>(p.out);
-  const WindowWeights &w = p.win;
+  const auto &w = WindowCoef<SH>::window(p);
   // trips start on rows congruent to 1 - M mod 4: where a run of whole trips
   // (y0 = 1 + run * H, H a multiple of 4) needs its first row
   constexpr int PH = (1 - M) & 3;
@@ -581,8 +609,47 @@ __device__ __forceinline__ int stream_sweep_window(const StreamParams &p, const 
       RowX n;
       n.ring_out = false;
       // a row beside the ring rows, or beside a ring column's value outside the window
-      const bool beside = (chk && (r == 1 || r == p.ny)) || (EDGE && __any_sync(0xffffffffu, c.ring_out));
-      if (((ph - t + 4 * M) & 3) < 2) {
+      const bool beside = (chk && (r == 1 || r == p.ny)) ||
+                          (EDGE && __any_sync(0xffffffffu, c.ring_out || (SH == 9 && (ym.ring_out || cur.ring_out))));
+      const bool exact = ((ph - t + 4 * M) & 3) < 2;
+      if constexpr (SH == 9) {
+        // the nine neighbours' columns: L, a, b, R of each row
+        if (exact) {
+          const Fx mL = shfl_up_fx(ym.xb), mR = shfl_down_fx(ym.xa), cL = shfl_up_fx(c.xb), cR = shfl_down_fx(c.xa),
+                   pL = shfl_up_fx(cur.xb), pR = shfl_down_fx(cur.xa);
+          n.a = window_sum<9>(w, q, {ym.xa, mL, ym.xb, c.xa, cL, c.xb, cur.xa, pL, cur.xb});
+          n.b = window_sum<9>(w, q, {ym.xb, ym.xa, mR, c.xb, c.xa, cR, cur.xb, cur.xa, pR});
+        }
+        const bool plain = (EDGE || chk) && beside;
+        if (!exact || plain) {
+          const double cL = __shfl_up_sync(0xffffffffu, c.b, 1), cR = __shfl_down_sync(0xffffffffu, c.a, 1);
+          const double pL = __shfl_up_sync(0xffffffffu, cur.b, 1), pR = __shfl_down_sync(0xffffffffu, cur.a, 1);
+          if (plain) {
+            const double mL = __shfl_up_sync(0xffffffffu, ym.b, 1), mR = __shfl_down_sync(0xffffffffu, ym.a, 1);
+            if (!exact) {
+              n.a = stencil_box(lk, mL, ym.a, ym.b, cL, c.a, c.b, pL, cur.a, cur.b);
+              n.b = stencil_box(lk, ym.a, ym.b, mR, c.a, c.b, cR, cur.a, cur.b, pR);
+            } else {
+              uint32_t da = 0, db = 0;
+              for (double u : {mL, ym.a, ym.b, cL, c.a, c.b, pL, cur.a, cur.b}) da |= (uint32_t)__double2hiint(u) - q.cref;
+              for (double u : {ym.a, ym.b, mR, c.a, c.b, cR, cur.a, cur.b, pR}) db |= (uint32_t)__double2hiint(u) - q.cref;
+              if (da >= w.lim) n.a = general_box_cell(lk, mL, ym.a, ym.b, cL, c.a, c.b, pL, cur.a, cur.b);
+              if (db >= w.lim) n.b = general_box_cell(lk, ym.a, ym.b, mR, c.a, c.b, cR, cur.a, cur.b, pR);
+              __syncwarp();
+            }
+          } else {
+            const Fx mL = shfl_up_fx(ym.xb), mR = shfl_down_fx(ym.xa);
+            const double ca[6] = {c.a, cL, c.b, cur.a, pL, cur.b}, cb[6] = {c.b, c.a, cR, cur.b, cur.a, pR};
+            n.a = window_head<kBoxHead>(w, q, {0, 1, 2}, {ym.xa, mL, ym.xb});
+            n.b = window_head<kBoxHead>(w, q, {0, 1, 2}, {ym.xb, ym.xa, mR});
+#pragma unroll
+            for (int u = 0; u < 6; ++u) {
+              n.a = fma_rn(lk.w[3 + u], ca[u], n.a);
+              n.b = fma_rn(lk.w[3 + u], cb[u], n.b);
+            }
+          }
+        }
+      } else if (exact) {
         const Fx L = shfl_up_fx(c.xb), R = shfl_down_fx(c.xa);
         n.a = window_exact(w, q, L, c.xb, ym.xa, c.xa, cur.xa);
         n.b = window_exact(w, q, c.xa, R, ym.xb, c.xb, cur.xb);
@@ -658,23 +725,27 @@ __device__ __forceinline__ int stream_sweep_window(const StreamParams &p, const 
   return y1;
 }
 
+__device__ __forceinline__ const Links<double> &chain_of(const WeightsD &k) { return k.l; }
+__device__ __forceinline__ const Box9<double> &chain_of(const WeightsD9 &k) { return k.b; }
+
 // A unit in windowed fixed point where its values allow it; elsewhere stretches
 // of rows by the general sweep: eight rows, four times as many while the window
 // keeps failing soon after, and all of them where a value is not positive.
-template <int M, bool EDGE, bool KEEP>
-__device__ __forceinline__ void stream_unit_window(const StreamParams &p, const WeightsD &k, long e0, int x0,
+template <int M, bool EDGE, bool KEEP, int SH>
+__device__ __forceinline__ void stream_unit_window(const StreamParams &p, const typename RowOf<double, SH>::W &k, long e0, int x0,
                                                    unsigned hold, bool live, bool st, int y0, int y1, float4 *ring) {
-  int stretch = p.win.lim ? 8 : y1;
+  const uint32_t lim = WindowCoef<SH>::window(p).lim;
+  int stretch = lim ? 8 : y1;
   while (y0 < y1) {
-    if (p.win.lim) {
-      const int y = stream_sweep_window<M, EDGE, KEEP>(p, k.l, e0, x0, hold, live, st, y0, y1, ring);
+    if (lim) {
+      const int y = stream_sweep_window<M, EDGE, KEEP, SH>(p, chain_of(k), e0, x0, hold, live, st, y0, y1, ring);
       if (y < 0) stretch = y1;
       else if (y - y0 >= 16) stretch = 8;
       y0 = max(y, y0);
     }
     if (y0 < y1) {
       const int ye = y0 + min(stretch, y1 - y0);
-      stream_sweep<double, M, EDGE, true, KEEP, 5>(p, k, e0, x0, hold, live, st, y0, ye, ring);
+      stream_sweep<double, M, EDGE, true, KEEP, SH>(p, k, e0, x0, hold, live, st, y0, ye, ring);
       y0 = ye;
       stretch = min(4 * stretch, 1 << 20);
     }
@@ -706,16 +777,17 @@ __device__ __forceinline__ void make_weights(const StreamParams &p, WeightsD *k)
 
 // Kernels whose units run in windowed fixed point.
 template <typename T, int M, bool IP, bool KEEP, int SH>
-constexpr bool kWindowed = std::is_same<T, double>::value && M <= 4 && IP && SH == 5;
+constexpr bool kWindowed = std::is_same<T, double>::value && M <= (SH == 5 ? 4 : 2) && IP;
 
 // Resident blocks per SM asked of the compiler (0: its own choice).  Windowed, M = 2:
 // five blocks of four warps (96 registers, some spilled in the rare branches)
-// measured faster than four or six (FP64 16384^2: 259, 252 and 255 GCells/s).
+// measured faster than four or six (FP64 16384^2: 259, 252 and 255 GCells/s); box:
+// four (144 at 16384^2; three 137, five 144; without the window 92).
 // Deep FP32 pipelines and the FP64 box: the occupancy they have had without
 // steady-trip registers on top (FP32 k = 12, 16384^2: 4126 GCells/s at 12 warps,
 // 3872 at 10).
 template <typename T, int M, bool IP, bool KEEP, int SH> constexpr int stream_blocks() {
-  if (kWindowed<T, M, IP, KEEP, SH>) return 7 - M;
+  if (kWindowed<T, M, IP, KEEP, SH>) return SH == 9 ? 4 : 7 - M;
   if (KEEP) return 0;
   if (std::is_same<T, float>::value && SH == 5) return M == 10 ? 13 : M == 12 ? 12 : 0;
   if (std::is_same<T, float>::value) return M == 8 ? 12 : 0;
@@ -751,9 +823,9 @@ __global__ void __launch_bounds__(32 * WarpsOf<T>::W, stream_blocks<T, M, IP, KE
   grid_dependency_wait();  // the pass before this one has finished and its rows are visible
   if constexpr (kWindowed<T, M, IP, KEEP, SH>) {
     if (edge)
-      stream_unit_window<M, true, KEEP>(p, k, e0, x0, hold, live, st, y0, y1, mine);
+      stream_unit_window<M, true, KEEP, SH>(p, k, e0, x0, hold, live, st, y0, y1, mine);
     else
-      stream_unit_window<M, false, KEEP>(p, k, e0, x0, hold, live, st, y0, y1, mine);
+      stream_unit_window<M, false, KEEP, SH>(p, k, e0, x0, hold, live, st, y0, y1, mine);
   } else if (edge)
     stream_sweep<T, M, true, IP, KEEP, SH>(p, k, e0, x0, hold, live, st, y0, y1, mine);
   else
@@ -823,10 +895,10 @@ static int stream_occupancy(j2d_dtype dt, int m, int shape) {
 StreamGeom stream_geometry(j2d_dtype dt, const GridDesc &g, int depth, int sms) {
   const int d = std::max(1, std::min(depth, stream_max_depth(dt)));
   const long warps = (long)stream_occupancy(dt, d, g.shape) * stream_warps(dt) * std::max(sms, 1);
-  return stream_geometry_warps(dt, g.nx, g.ny, depth, warps, g.shape);
+  return stream_geometry_warps(dt, g.nx, g.ny, depth, warps);
 }
 
-StreamGeom stream_geometry_warps(j2d_dtype dt, int nx, int ny, int depth, long warps, int shape) {
+StreamGeom stream_geometry_warps(j2d_dtype dt, int nx, int ny, int depth, long warps) {
   StreamGeom q;
   const int V = dt == J2D_F64 ? 2 : 4;
   q.depth = std::max(1, std::min(depth, stream_max_depth(dt)));
@@ -840,7 +912,7 @@ StreamGeom stream_geometry_warps(j2d_dtype dt, int nx, int ny, int depth, long w
   // 4096^2: 2764 against 2175 with 32M).
   warps = std::max(warps, 1L);
   const int hmin = (dt == J2D_F64 ? 32 : 16) * q.depth;
-  if (dt == J2D_F64 && shape == 5) {
+  if (dt == J2D_F64) {
     // Whole waves of units, up to eight with runs of at least 44M rows (k = 2,
     // 8192^2: 212, 233, 236, 238, 239 and 235 GCells/s with 1, 2, 3, 4, 6 and 8
     // waves, 16384^2: 258 with 6, 259 with 8, 258 with 16); one wave for
@@ -893,6 +965,8 @@ cudaError_t launch_stream_pass(j2d_dtype dt, const void *in, void *out, const Gr
   p.status = status;
   for (int i = 0; i < 9; ++i) p.w[i] = g.w[i];
   p.win = WindowWeights{};
+  p.win9 = WindowWeightsN<9>{};
+  if (dt == J2D_F64 && g.shape == 9) p.win9 = window_weights(box_chain<double>(g.w).w);
   if (dt == J2D_F64 && g.shape == 5) p.win = window_weights({g.w[0], g.w[1], g.w[2], g.w[3], g.w[4]});
   StreamFn fn = stream_fn(dt, q.depth, ipath, keep != nullptr, g.shape);
   if (!fn || m < 1 || m > q.depth) return cudaErrorInvalidValue;

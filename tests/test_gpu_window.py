@@ -134,3 +134,35 @@ def test_window_states(fname):
             assert np.array_equal(plan.to_host(states[t]), plan.to_host(nxt)), (depth, t)
             cur = nxt
         plan.close()
+
+
+BOX_WEIGHTS = {
+    "even": [1 / 9] * 9,
+    "spread3": [0.18, 0.03, 0.09, 0.12, 0.15, 0.11, 0.07, 0.17, 0.08],
+    "spread5": [0.25, 0.008, 0.09, 0.12, 0.15, 0.11, 0.07, 0.132, 0.07],
+    "spread7": [0.25, 0.0018, 0.09, 0.12, 0.15, 0.11, 0.07, 0.138, 0.07],
+    "zero": [0.125, 0.125, 0.125, 0.125, 0.0, 0.125, 0.125, 0.125, 0.125],
+    "negative": [0.2, 0.1, -0.05, 0.15, 0.2, 0.1, 0.1, 0.1, 0.1],
+}
+
+
+@pytest.mark.parametrize("fname", ["uniform", "spikes", "ring", "zero_ring", "ramp", "wide", "tiny", "huge", "short"])
+@pytest.mark.parametrize("nx,ny", [(1, 1), (3, 2), (61, 70), (124, 129), (187, 301)])
+def test_window_box_fields(fname, nx, ny):
+    u = field(fname, nx, ny)
+    w = np.array(BOX_WEIGHTS["spread3"])
+    for steps in (1, 4, 5):
+        ref = run(u, w, nx, ny, steps, "onestep", 0)
+        got = run(u, w, nx, ny, steps, "stream", 2)
+        assert np.array_equal(got, ref), "%d steps: %d cells differ" % (steps, np.count_nonzero(got != ref))
+
+
+@pytest.mark.parametrize("wname", sorted(BOX_WEIGHTS))
+def test_window_box_weights(wname):
+    nx, ny = 130, 203
+    w = np.array(BOX_WEIGHTS[wname])
+    for fname in ("spikes", "short"):
+        u = field(fname, nx, ny)
+        ref = run(u, w, nx, ny, 4, "onestep", 0)
+        got = run(u, w, nx, ny, 4, "stream", 2)
+        assert np.array_equal(got, ref), "%s: %d cells differ" % (fname, np.count_nonzero(got != ref))
