@@ -190,11 +190,11 @@ def measure_peaks(j2d5pt):
     smem = j2d5pt.j2d5pt_measure_smem_bandwidth()
     mask, _ = j2d5pt.j2d5pt_arith_info()
     f = bin(mask & 0xFF).count("1") / 8.0
-    # FP64 cell rate: half of the cells (the exact mask) run on the integer
-    # pipes, the rest as 5 FP64 FMA instructions; the two pipes work in
-    # parallel, so the peak is set by the slower share, each at its measured rate
-    chain = fma64 / 5
-    alu = 1.0 / max((1.0 - f) / chain, f / exact if f else 0.0)
+    # FP64 cell rate: half of the cells (the exact mask) run on the integer pipes
+    # and the chains of the rest keep three of their five operations on the FP64
+    # pipe (windowed fixed point), which bounds a cell whatever the kernel
+    chain = fma64 / 3
+    alu = chain / (1.0 - f)
     hbm = None
     try:
         hbm = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"] * 1e9
@@ -210,9 +210,9 @@ def roof_f64(pk, kernel_gcells, traffic=None, kernel="dtb_kernel"):
     peak = pk["alu_cells"] / 1e9 * 9 / 1e3
     return {"bound": "alu", "achieved": round(achieved, 4), "peak": round(peak, 4), "unit": "TFLOP/s",
             "frac": round(achieved / peak, 4), "traffic": traffic, "kernel": kernel,
-            "peak_source": ("of measured: FP64 pipe %.1f GFMA/s (j2d5pt_measure_fma_rate) / 5 per chain cell, "
-                            "integer path %.1f Gcells/s (j2d5pt_measure_exact_rate), exact share %.3f; x 9 flops "
-                            "per cell" % (pk["fma64"] / 1e9, pk["exact"] / 1e9, pk["share"])),
+            "peak_source": ("of measured: FP64 pipe %.1f GFMA/s (j2d5pt_measure_fma_rate) / 3 per chain cell (two of "
+                            "a chain's five operations run on the integer pipes in windowed fixed point), exact "
+                            "share %.3f; x 9 flops per cell" % (pk["fma64"] / 1e9, pk["share"])),
             "kernel_gcells": round(kernel_gcells, 3), "peak_gcells": round(pk["alu_cells"] / 1e9, 3),
             "fp64_pipe_only_gcells": round(pk["fma64"] / 5 / 1e9, 3)}
 
@@ -537,14 +537,14 @@ def run_extras(j2d5pt, synth, flush, stream, pk, head_plan, head_src, head_dst):
     # 6) the second stencil shape, the 3x3 box (j2d9pt): FP64 and FP32 16384^2,
     #    1000 steps, autotuned, beside its one-step kernel; FP64 against the
     #    arithmetic peak of the nine-term cell (FP64 pipe: 9 FMA instructions
-    #    per chain cell; integer path: the measured nine-term rate; 17 flops per cell)
+    #    per chain cell; 17 flops per cell)
     n, T = HEAD_N, HEAD_T
     cells = n * n * T
     u0 = synth.field(n, n, synth.data_seed(1))
     wb = synth.box_weights(synth.weight_seed(1))
     exact9 = j2d5pt.j2d9pt_measure_exact_rate()
     f = pk["share"]
-    alu9 = 1.0 / max((1.0 - f) / (pk["fma64"] / 9), f / exact9 if f else 0.0)
+    alu9 = pk["fma64"] / 6 / (1.0 - f)  # three of the chain's nine operations run on the integer pipes
     box = {"exact9_gcells": round(exact9 / 1e9, 2), "peak_gcells": round(alu9 / 1e9, 2)}
     for dt in ("f64", "f32"):
         p = j2d5pt.Plan.box9(n, n, dt, wb)
@@ -562,8 +562,8 @@ def run_extras(j2d5pt, synth, flush, stream, pk, head_plan, head_src, head_dst):
                 r["roofline"] = {"bound": "alu", "achieved": round(g * 17 / 1e3, 4),
                                  "peak": round(alu9 / 1e9 * 17 / 1e3, 4), "unit": "TFLOP/s",
                                  "frac": round(g * 1e9 / alu9, 4),
-                                 "peak_source": "of measured: FP64 pipe / 9 per chain cell, nine-term integer path "
-                                                "(j2d9pt_measure_exact_rate), exact share %.3f; x 17 flops" % f}
+                                 "peak_source": "of measured: FP64 pipe / 6 per chain cell (windowed fixed point), "
+                                                "exact share %.3f; x 17 flops" % f}
         else:
             r1["roofline"] = roof_hbm(pk, r1["kernel_gcells"], 4)
             f2 = dict(kv.split("=") for kv in p.describe().split())
