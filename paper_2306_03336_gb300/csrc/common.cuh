@@ -39,12 +39,13 @@ __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fm
 // The FP64 pipe takes an FMA of three vector registers every 64 clocks per
 // warp and SM quarter, but a multiply, an add, or an FMA with a constant-bank
 // or uniform-register operand only every 76 (597 against 502 G/s over the
-// chip at 1.99 GHz, whatever the number of warps).  So FP64 kernels hold
-// their weights in vector registers (vreg(): a shuffle by the lane's own index,
-// which the compiler cannot prove uniform) and take the chain's first product
-// as an FMA that adds -0.0, which rounds exactly as the multiply does, signs
-// of zeros included; the -0.0 is a vector register too (nz), or the compiler
-// would turn the FMA back into a multiply.
+// chip at 1.99 GHz, whatever the number of warps).  So the five-point FP64
+// stream kernels and the windowed adjoint hold their weights in vector registers
+// (vreg(): a shuffle by the lane's own index, which the compiler cannot prove
+// uniform; elsewhere the integer path binds and the registers are better spent)
+// and take the chain's first product as an FMA that adds -0.0, which rounds
+// exactly as the multiply does, signs of zeros included; the -0.0 is a vector
+// register too (nz), or the compiler would turn the FMA back into a multiply.
 __device__ __forceinline__ double vreg(double v) { return __shfl_sync(0xffffffffu, v, threadIdx.x & 31); }
 __device__ __forceinline__ float vreg(float v) { return v; }  // FP32: no such difference
 template <typename T> __device__ __forceinline__ Links<T> vreg_links(const Links<T> &a) {

@@ -29,10 +29,11 @@
 // Every cell is evaluated exactly as the one-step kernel evaluates it: FP32 by
 // the chain of stencil() in common.cuh (here two cells per paired FP32 multiply
 // and fused multiply-add, each element rounded as the scalar instruction
-// rounds it), FP64 by stencil_cell() with the integer path on the same cells.
+// rounds it), FP64 by stencil_cell() with the integer path on the same cells, or the
+// same values in windowed fixed point where a unit's values allow it (window.cuh).
 // So the results are bit-identical to every other kernel of the library.
 //
-// One launch per pass (the passes of a run are ordered on the stream; a run of
+// One launch per pass (a pass waits for the one before it; a run of
 // S steps is ceil(S / M) passes, the first one taking the remainder), with
 // several waves of (band, run) units so that the block scheduler balances the
 // SMs.  Per cell update HBM carries 2 * sizeof(T) * (1 + overlap) / M bytes.

@@ -17,7 +17,7 @@
 // for every exponent spread h up to 5 and, for weights of a comparable sum, 7.
 // k = 7 for h <= 4, else 3, so k + h <= 11 = kExactGuard, so every windowed cell satisfies the integer path's contract and
 // its correctly rounded sum is the result stencil_exact() gives: bit for bit the
-// same, at about 50 instructions per cell instead of 166 (315 against 150
+// same, at about 50 instructions per cell instead of 166 (350 against 150
 // Gcells/s measured alone at 1.99 GHz, register operands).
 //
 // The FMA chain's first product and its first FMA are evaluated the same way
