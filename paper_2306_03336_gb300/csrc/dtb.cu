@@ -1885,8 +1885,10 @@ DtbConfig dtb_choose(j2d_dtype dt, const std::vector<GridDesc> &grids, int sms, 
     // FP64 box grids whose weights fit the windowed fixed point: the stream schedule
     // at every size (4096^2: 150 us a step against 231 for the skewed tiles,
     // 2048x1536: 42 against 63, 512^2: 16 against 29; fields of both signs, which no
-    // window takes, 330 against 319, 90 against 86, 28 against 37)
-    else if (rq.windowed) algo = J2D_ALGO_STREAM;
+    // window takes, 330 against 319, 90 against 86, 28 against 37).  Not for four or
+    // five steps: the first pass over noise takes the general sweep (1500^2, four
+    // steps: 277 us against 237; eight: 393 against 486)
+    else if (rq.windowed && rq.steps >= 6) algo = J2D_ALGO_STREAM;
     else if (fits && (dt == J2D_F64 || (single && rq.adjoint))) algo = J2D_ALGO_RESIDENT;
     // grids too large for the chip: the stream schedule for FP32 (16384^2:
     // 4254 GCells/s against 1950 for the best shared-memory schedule; the box
@@ -1895,7 +1897,8 @@ DtbConfig dtb_choose(j2d_dtype dt, const std::vector<GridDesc> &grids, int sms, 
     // signs, which no window takes, 4096^2: 91 against 86), and for large FP64
     // box grids
     else if (single && !rq.adjoint &&
-             (dt == J2D_F32 || grids[0].shape == 5 || (long)grids[0].nx * grids[0].ny >= (8192L << 13)))
+             (dt == J2D_F32 || (grids[0].shape == 5 && rq.steps >= 6) ||
+              (long)grids[0].nx * grids[0].ny >= (8192L << 13)))
       algo = J2D_ALGO_STREAM;
     // FP64 adjoint runs of larger grids: the one-step kernel (4096^2: 98 us a step
     // against 134 for the tiles, 2304x1700: 28 against 49; fields of both signs 163
@@ -1921,9 +1924,13 @@ DtbConfig dtb_choose(j2d_dtype dt, const std::vector<GridDesc> &grids, int sms, 
   }
   // FP32: eight steps a pass for large five-point grids (16384^2: 4660 GCells/s, 4260
   // with six), six for smaller ones, whose units are short (2048x1536: 2.3 against
-  // 1.9 us a step), and for the box (16384^2: 2445 against 2744)
-  if (algo == J2D_ALGO_STREAM && rq.depth <= 0)
-    c.depth = dt == J2D_F64 ? 2 : (long)grids[0].nx * grids[0].ny >= (3200L * 3200) && grids[0].shape == 5 ? 8 : 6;
+  // 1.9 us a step), and for the box (16384^2: 2445 against 2744); a run of seven or
+  // eight steps is one pass of eight (box 6000x1800: 83 us in two passes, 77 in one)
+  if (algo == J2D_ALGO_STREAM && rq.depth <= 0) {
+    const bool one8 = rq.steps == 7 || rq.steps == 8;
+    const bool large = (long)grids[0].nx * grids[0].ny >= 3200L * 3200 && grids[0].shape == 5;
+    c.depth = dt == J2D_F64 ? 2 : large || one8 ? 8 : 6;
+  }
   if (algo == J2D_ALGO_SKEWED) {
     c.rows = dtb_rows_max_skew(dt, smem_optin);
     if (rq.depth <= 0) c.depth = dt == J2D_F64 ? 8 : 16;
