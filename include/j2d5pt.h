@@ -78,12 +78,14 @@ typedef enum {
                             rows, advancing k steps per pass as a pipeline held in registers
                             (step t of row i-t as row i arrives); one launch per pass, no shared
                             memory.  k in {4, 6, 8, 10, 12} for FP32, {2, 3, 4, 6} for FP64
-                            (J2D_ERR_ARG otherwise; default 8, or 6 below 3200^2 cells, and 2);
+                            (J2D_ERR_ARG otherwise; default 8, or 6 below 3200^2 cells unless
+                            the run has 7 or 8 steps, and 2);
                             box plans: {4, 6, 8} for FP32, {2, 3, 4} for FP64 (default 6 and 2).  Forward runs of single
                             grids only (adjoint runs and batches take TILES).  AUTO takes it for
-                            FP32 grids, for FP64 grids too large for the chip and for FP64
-                            box grids (weights within about 32 times of each other, or
-                            8192^2 cells or more). */
+                            FP32 grids and, in runs of six steps or more, for FP64 grids
+                            too large for the chip and FP64 box grids whose weights lie
+                            within about 32 times of each other (FP64 grids of 8192^2
+                            cells or more: from four steps on). */
 } j2d_algo;
 
 /* Plan options (j2d5pt_set_option / j2d5pt_get_option). */
@@ -134,9 +136,7 @@ j2d_status j2d5pt_plan_batched(j2d5pt_plan_t *plan, int count, const int *nx, co
  * j2d5pt_run / j2d5pt_run_host / j2d5pt_autotune and the option, layout,
  * describe, timing and status calls; its algorithms are J2D_ALGO_ONESTEP,
  * J2D_ALGO_SKEWED and J2D_ALGO_STREAM (any other choice runs the skewed
- * tiles; AUTO takes the stream schedule for FP32 grids and, when the weights
- * lie within about 32 times of each other or the grid has 8192^2 cells or
- * more, for FP64 grids).  The adjoint,
+ * tiles; AUTO takes the stream schedule as J2D_ALGO_STREAM above says).  The adjoint,
  * weight-gradient and j2d5pt_set_weights calls return J2D_ERR_UNSUPPORTED.
  * FP64 cells are evaluated as j2d5pt_arith_info describes, with the nine
  * terms: the FMA chain takes the product of the (y-1, x) term, then the
