@@ -91,7 +91,10 @@ typedef enum {
 /* Plan options (j2d5pt_set_option / j2d5pt_get_option). */
 typedef enum {
   J2D_OPT_ALGO = 0,       /* j2d_algo */
-  J2D_OPT_DEPTH = 1,      /* temporal depth k (steps per on-chip visit) for BANDS / TILES / SKEWED */
+  J2D_OPT_DEPTH = 1,      /* temporal depth k (steps per on-chip visit) for BANDS / TILES / SKEWED / STREAM.
+                             With AUTO and a depth other than {4, 6, 8} for FP32 or 2 for FP64, grids
+                             that fit on chip stay there and larger FP64 grids below 8192^2 cells
+                             take TILES (box plans: SKEWED) */
   J2D_OPT_TILE_WX = 2,    /* TILES / SKEWED: warp strips across a CTA tile (16 / WX down) */
   J2D_OPT_CTAS = 3,       /* persistent grid size (0 = one CTA per SM) */
   J2D_OPT_TIMEOUT_MS = 4, /* device-side wait limit in milliseconds (default 2000) */

@@ -1873,6 +1873,14 @@ DtbConfig dtb_choose(j2d_dtype dt, const std::vector<GridDesc> &grids, int sms, 
   const int sw = 32 * vec_of(dt);
   int algo = rq.algo;
   const bool single = grids.size() == 1;
+  // A depth the caller set is the depth of whatever AUTO takes, so AUTO takes the
+  // stream schedule beside the schedules that ran there before it only where it has
+  // that depth and is the faster one (microseconds, before and stream: FP64 2304x1700
+  // x 48, depth 3: 1901 and 1877, 4: 1941 and 2447, 6: 1873 and 2859; box 4096^2 x 24,
+  // depth 3: 5465 and 7230; FP32 200x120 x 48, depth 8: 103 and 88, 10: 103 and 134)
+  const bool depth_streams =
+      rq.depth <= 0 ||
+      (dt == J2D_F64 ? rq.depth == 2 : rq.depth <= 8 && stream_depth_ok(dt, rq.depth, grids[0].shape));
   int m = 0;
   const bool fits = single ? resident_fit(grids[0], sw, c.ctas, c.rows, &m)
                            : !rq.adjoint && groups_fit(grids, sw, c.ctas, c.rows);
@@ -1888,8 +1896,8 @@ DtbConfig dtb_choose(j2d_dtype dt, const std::vector<GridDesc> &grids, int sms, 
     // window takes, 330 against 319, 90 against 86, 28 against 37).  Not for four or
     // five steps: the first pass over noise takes the general sweep (1500^2, four
     // steps: 277 us against 237; eight: 393 against 486)
-    else if (rq.windowed && rq.steps >= 6) algo = J2D_ALGO_STREAM;
-    else if (fits && (dt == J2D_F64 || (single && rq.adjoint))) algo = J2D_ALGO_RESIDENT;
+    else if (rq.windowed && rq.steps >= 6 && depth_streams) algo = J2D_ALGO_STREAM;
+    else if (fits && (dt == J2D_F64 || (single && (rq.adjoint || !depth_streams)))) algo = J2D_ALGO_RESIDENT;
     // grids too large for the chip: the stream schedule for FP32 (16384^2:
     // 4254 GCells/s against 1950 for the best shared-memory schedule; the box
     // 2578 against 1418) and five-point FP64 (16384^2: 259 against 162 for the
@@ -1897,7 +1905,7 @@ DtbConfig dtb_choose(j2d_dtype dt, const std::vector<GridDesc> &grids, int sms, 
     // signs, which no window takes, 4096^2: 91 against 86), and for large FP64
     // box grids
     else if (single && !rq.adjoint &&
-             (dt == J2D_F32 || (grids[0].shape == 5 && rq.steps >= 6) ||
+             (dt == J2D_F32 || (grids[0].shape == 5 && rq.steps >= 6 && depth_streams) ||
               (long)grids[0].nx * grids[0].ny >= (8192L << 13)))
       algo = J2D_ALGO_STREAM;
     // FP64 adjoint runs of larger grids: the one-step kernel (4096^2: 98 us a step
