@@ -83,9 +83,10 @@ typedef enum {
                             box plans: {4, 6, 8} for FP32, {2, 3, 4} for FP64 (default 6 and 2).  Forward runs of single
                             grids only (adjoint runs and batches take TILES).  AUTO takes it for
                             FP32 grids and, in runs of six steps or more, for FP64 grids
-                            too large for the chip and FP64 box grids whose weights lie
-                            within about 32 times of each other (FP64 grids of 8192^2
-                            cells or more: from four steps on). */
+                            too large for the chip (unless their weights are all positive
+                            and spread over more than about 100 times) and FP64 box grids
+                            whose weights lie within about 32 times of each other (FP64
+                            grids of 8192^2 cells or more: from four steps on). */
 } j2d_algo;
 
 /* Plan options (j2d5pt_set_option / j2d5pt_get_option). */

@@ -1,6 +1,7 @@
 // api.cu -- the C ABI (include/j2d5pt.h): plans, validation, workspace,
 // dispatch to the one-step and temporally blocked kernels, host end-to-end
 // runs, status reporting.
+#include <cfloat>
 #include <cmath>
 #include <cstdint>
 #include <cstdarg>
@@ -284,6 +285,18 @@ extern "C" j2d_status j2d5pt_get_option(j2d5pt_plan_t p, j2d_option opt, long *v
   return J2D_OK;
 }
 
+// What the FP64 integer path can do with the plan's weights (one grid).
+static WeightClass weight_class(j2d5pt_plan_t p) {
+  const GridDesc &g = p->grids[0];
+  const int n = g.shape;  // five or nine weights
+  if (!int_path_of(p)) return WEIGHTS_CHAIN;
+  for (int i = 0; i < n; ++i)
+    if (!(g.w[i] >= DBL_MIN)) return WEIGHTS_CHAIN;  // negative, zero or subnormal: every cell takes the chain
+  const uint32_t lim = n == 9 ? window_weights(box_chain<double>(g.w).w).lim
+                              : window_weights({g.w[0], g.w[1], g.w[2], g.w[3], g.w[4]}).lim;
+  return lim ? WEIGHTS_WINDOWED : WEIGHTS_POSITIVE;
+}
+
 // Resolve the configuration a run will use.
 static DtbConfig resolve(j2d5pt_plan_t p, long steps, bool adj) {
   DtbRequest rq;
@@ -294,8 +307,7 @@ static DtbConfig resolve(j2d5pt_plan_t p, long steps, bool adj) {
   rq.steps = steps;
   rq.adjoint = adj;
   rq.sweep_steps = p->opt_sweep_steps;
-  const GridDesc &g = p->grids[0];
-  rq.windowed = int_path_of(p) && g.shape == 9 && window_weights(box_chain<double>(g.w).w).lim != 0;
+  rq.weights = weight_class(p);
   return dtb_choose(p->dtype, p->grids, p->sms, p->smem_optin, rq);
 }
 

@@ -1896,16 +1896,19 @@ DtbConfig dtb_choose(j2d_dtype dt, const std::vector<GridDesc> &grids, int sms, 
     // window takes, 330 against 319, 90 against 86, 28 against 37).  Not for four or
     // five steps: the first pass over noise takes the general sweep (1500^2, four
     // steps: 277 us against 237; eight: 393 against 486)
-    else if (rq.windowed && rq.steps >= 6 && depth_streams) algo = J2D_ALGO_STREAM;
+    else if (grids[0].shape == 9 && rq.weights == WEIGHTS_WINDOWED && rq.steps >= 6 && depth_streams) algo = J2D_ALGO_STREAM;
     else if (fits && (dt == J2D_F64 || (single && (rq.adjoint || !depth_streams)))) algo = J2D_ALGO_RESIDENT;
     // grids too large for the chip: the stream schedule for FP32 (16384^2:
     // 4254 GCells/s against 1950 for the best shared-memory schedule; the box
     // 2578 against 1418) and five-point FP64 (16384^2: 259 against 162 for the
     // tiles; 4096^2: 193 against 145; 2304x1700: 146 against 97; fields of both
-    // signs, which no window takes, 4096^2: 91 against 86), and for large FP64
-    // box grids
+    // signs, which no window takes, 4096^2: 91 against 86; every cell a chain, as with
+    // a zero or negative weight or without the integer path: 100 against 87), and
+    // for large FP64 box grids.  Positive weights without a window stay with the
+    // tiles below 8192^2 (spread 2^10, 3001x4099: 121 and 115 GCells/s, tiles and
+    // stream, 4096^2: 140 and 126)
     else if (single && !rq.adjoint &&
-             (dt == J2D_F32 || (grids[0].shape == 5 && rq.steps >= 6 && depth_streams) ||
+             (dt == J2D_F32 || (grids[0].shape == 5 && rq.weights != WEIGHTS_POSITIVE && rq.steps >= 6 && depth_streams) ||
               (long)grids[0].nx * grids[0].ny >= (8192L << 13)))
       algo = J2D_ALGO_STREAM;
     // FP64 adjoint runs of larger grids: the one-step kernel (4096^2: 98 us a step

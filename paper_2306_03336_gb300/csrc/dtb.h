@@ -10,6 +10,11 @@ struct j2d5pt_plan_s;
 
 namespace j2d {
 
+// What the FP64 integer path can do with a plan's weights: nothing (the path is off
+// or a weight is not positive normal, so every cell is an FMA chain), exact sums
+// cell by cell, or exact sums in windowed fixed point (window.cuh).
+enum WeightClass { WEIGHTS_CHAIN, WEIGHTS_POSITIVE, WEIGHTS_WINDOWED };
+
 struct DtbRequest {
   int algo = J2D_ALGO_AUTO;
   int depth = 0;
@@ -18,7 +23,7 @@ struct DtbRequest {
   long steps = 0;
   bool adjoint = false;
   int sweep_steps = 2;  // TILES, FP32 forward: steps per sweep (J2D_OPT_SWEEP_STEPS)
-  bool windowed = false;  // FP64 box: the plan's weights fit windowed fixed point (window.cuh) and the integer path is on
+  WeightClass weights = WEIGHTS_CHAIN;  // FP64: what the integer path can do with the plan's weights
 };
 
 // Everything one temporally blocked run needs.
