@@ -189,7 +189,8 @@ j2d_status j2d5pt_run_host(j2d5pt_plan_t plan, const void *h_in, void *h_out, lo
  * state t (1 <= t <= steps, ring included) is written at states + (t-1) *
  * (ny+2) * pitch elements.  Bit-identical to `steps` chained calls of
  * j2d5pt_run(plan, ., ., 1, stream).  With J2D_ALGO_AUTO FP64
- * grids too large for the chip take the stream passes, others the one-step
+ * grids of 8 M cells or more whose weights have a window (see
+ * J2D_ALGO_STREAM) take the stream passes from six states on, others the one-step
  * kernel, one launch per state (it writes every state anyway); a plan set to a
  * temporally blocked algorithm stores each state from its one persistent
  * launch (the skewed and two-step FP32 schedules run as single-step tiles

@@ -638,12 +638,17 @@ extern "C" j2d_status j2d5pt_run_states(j2d5pt_plan_t p, const void *in, void *s
   p->ran = true;
   cudaError_t e;
   if ((e = launch_ring_copy(p->dtype, in, states, g, s, steps, se)) != cudaSuccess) return cuda_fail(e, "run_states: rings");
-  // AUTO keeps the states of FP64 grids too large for the chip with the stream
-  // passes (4096^2: 101 us a state against 132 for the one-step kernel; fields of
-  // both signs, which no window takes, 181 against 171), of others with the one-step
-  // kernel, which writes every state anyway
+  // AUTO keeps states with the one-step kernel, which writes every state anyway, but
+  // for FP64 grids of 8 M cells and more whose weights have a window, which take
+  // the stream passes.  Microseconds a state, one-step and stream: 4096^2, noise 132 and
+  // 97, smooth positive fields 132 and 87, fields of both signs, which no window
+  // takes, 171 and 179; 2304x1700, six states, 37 and 45, 37 and 28, 49 and 53; weights without
+  // a window, 4096^2: 135 and 140, with a zero or negative one 156 and 169.
   DtbConfig c = resolve(p, steps, false);
-  if (p->opt_algo == J2D_ALGO_AUTO && !(c.algo == J2D_ALGO_STREAM && p->dtype == J2D_F64)) c.algo = J2D_ALGO_ONESTEP;
+  if (p->opt_algo == J2D_ALGO_AUTO &&
+      !(c.algo == J2D_ALGO_STREAM && p->dtype == J2D_F64 && weight_class(p) == WEIGHTS_WINDOWED &&
+        (long)g.nx * g.ny >= 8L << 20))
+    c.algo = J2D_ALGO_ONESTEP;
   if (c.algo == J2D_ALGO_ONESTEP) {
     const void *src = in;
     for (long t = 0; t < steps; ++t) {

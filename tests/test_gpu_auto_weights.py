@@ -39,3 +39,23 @@ def test_large_grids_and_short_spreads_keep_the_stream():
     p = j2d5pt.Plan(8192, 8192, "f64", w)
     assert "algo=stream " in p.describe()
     p.close()
+
+
+@pytest.mark.parametrize("nx,ny,w,launches", [
+    (2304, 1700, FIVE[0][0], 8),  # below 8 M cells: the one-step kernel
+    (4096, 2100, FIVE[0][0], 4),  # a window: passes of two steps
+    (4096, 2100, FIVE[1][0], 8),  # positive without a window
+    (4096, 2100, FIVE[4][0], 8)])  # a zero weight
+def test_kept_states_route(nx, ny, w, launches):
+    import torch
+    steps = 8
+    p = j2d5pt.Plan(nx, ny, "f64", np.array(w))
+    src, one = p.to_device(synth.field(nx, ny, 52)), p.empty()
+    states = p.empty_states(steps)
+    before = j2d5pt.j2d5pt_kernel_launches()
+    p.run_states(src, states, steps)
+    assert j2d5pt.j2d5pt_kernel_launches() - before == 1 + launches  # the rings of all states in one
+    p.set("algo", "onestep").run(src, one, steps)
+    p.sync()
+    assert torch.equal(p.view(states[steps - 1]), p.view(one))
+    p.close()
