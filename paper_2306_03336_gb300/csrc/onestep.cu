@@ -127,11 +127,50 @@ __device__ __forceinline__ bool adjoint_item_window(const double (&t)[ROWS + 2][
   return true;
 }
 
+// Bits of a value's magnitude, enough of them to tell a finite value from an infinity or
+// a NaN.
+__device__ __forceinline__ int magnitude(double v) { return __double2hiint(v) & 0x7fffffff; }
+__device__ __forceinline__ int magnitude(float v) { return __float_as_int(v) & 0x7fffffff; }
+template <typename T> constexpr int kInfinite = sizeof(T) == 8 ? 0x7ff00000 : 0x7f800000;
+
+// The cells that onestep_kernel's zero links spoil beside an infinity or a NaN (zero times
+// it is NaN), written again for one lane's vector in rows [ya, yb).  Forward: ring
+// cells are held.  Adjoint: no cell takes anything from the ring, and a ring cell adds
+// its one interior neighbour to its value.  Slow, out of line, and run only for
+// items that reach the ring and store an infinity or a NaN.
+template <typename T, bool ADJ>
+__device__ __noinline__ void nonfinite_item(const T *__restrict__ in, T *__restrict__ out, long pitch, long pc0, int xl0,
+                                            int ya, int yb, int nx, int ny, Weights<T> w, int ipath) {
+  auto ring = [&](int x, int y) { return x < 1 || x > nx || y < 1 || y > ny; };
+  for (int y = ya; y < yb; ++y)
+    for (int v = 0; v < VecOf<T>::V; ++v) {
+      const int x = xl0 + v;
+      if (x < 0 || x > nx + 1) continue;
+      const long e = (long)y * pitch + pc0 + v;
+      if (!ADJ) {
+        if (ring(x, y)) out[e] = in[e];
+        continue;
+      }
+      Links<T> a = cell_links<T, true>(2, 2, 4, 4, w);
+      const Links<T> interior = a;
+      if (ring(x, y)) a.c = T(1);
+      const T xm = ring(x - 1, y) ? T(0) : in[e - 1], xp = ring(x + 1, y) ? T(0) : in[e + 1];
+      const T ym = ring(x, y - 1) ? T(0) : in[e - pitch], yp = ring(x, y + 1) ? T(0) : in[e + pitch];
+      if constexpr (std::is_same<T, double>::value)
+        out[e] = stencil_cell(a, exact_weights(interior), !ring(x, y) && exact_cell(x, y, ipath != 0), xm, xp, ym, in[e], yp);
+      else
+        out[e] = stencil(a, xm, xp, ym, in[e], yp);
+    }
+}
+
 // WG (adjoint only): also accumulate the weight gradient of this step,
 // sum over interior cells of in[i] * u[nbr_d(i)] (in = lam_t+1), into one
 // partial sum per block, reduced in a fixed order.
+// Two blocks an SM (128 registers) are asked of the compiler where its own choice exceeds
+// them by a few: FP32 adjoint (4096^2 36 -> 34 us a step, no spills) and the fused FP64
+// pass (146 registers, 363 us a step at 4096^2 against 270).
 template <typename T, bool ADJ, int ROWS, bool WG = false>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 && ADJ ? 2 : 0) onestep_kernel(const T *__restrict__ in, T *__restrict__ out, long pitch,
+__global__ void __launch_bounds__(256, WG || (ADJ && sizeof(T) == 4) ? 2 : 0) onestep_kernel(const T *__restrict__ in, T *__restrict__ out, long pitch,
                                                       int off, int nx, int ny, Weights<T> w, int ipath,
                                                       WindowWeights win, const T *__restrict__ uw = nullptr,
                                                       double *__restrict__ partials = nullptr) {
@@ -191,12 +230,15 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 && ADJ ? 2 : 0) onestep_ke
     }
   }
 
+  const int xw0 = (int)((it % ncs) * 32 * V) - off;
+  const bool edge = xw0 <= 1 || xw0 + 32 * V > nx || y0 <= 1 || y0 + ROWS > ny;  // the item reaches the ring
+  int top = 0;  // then: the largest magnitude it stores
   const bool lval = live && (xl0 - 1 >= 0) && (xl0 - 1 <= nx + 1);
   const bool rval = live && (xl0 + V <= nx + 1);
   bool done = false;  // the item's results are stored already
   if constexpr (kWindowed) {
     if (ipath && win.lim)
-      done = adjoint_item_window<ROWS>(t, in, out, pitch, pc0, (int)((it % ncs) * 32 * V) - off, y0, nx, ny, wl, win);
+      done = adjoint_item_window<ROWS>(t, in, out, pitch, pc0, xw0, y0, nx, ny, wl, win);
     if (!WG && done) continue;
   }
   Links<T> cw[V];  // links of this thread's columns on rows away from the ring
@@ -237,6 +279,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 && ADJ ? 2 : 0) onestep_ke
       }
     }
     if (live) *reinterpret_cast<VT *>(out + (long)y * pitch + pc0) = pack(o, (VT *)nullptr);
+    if (edge) {
+#pragma unroll
+      for (int v = 0; v < V; ++v) top = max(top, magnitude(o[v]));
+    }
     }
     if constexpr (WG) {
       T ul = __shfl_up_sync(0xffffffffu, uu[r + 1][V - 1], 1);
@@ -258,6 +304,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 && ADJ ? 2 : 0) onestep_ke
       }
     }
   }
+  if (edge && __any_sync(0xffffffffu, top >= kInfinite<T>) && live)
+    nonfinite_item<T, ADJ>(in, out, pitch, pc0, xl0, y0, min(y0 + ROWS, H), nx, ny, w, ipath);
   }
   if constexpr (WG) block_partials(acc, partials);
 }
