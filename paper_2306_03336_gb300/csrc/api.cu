@@ -641,7 +641,7 @@ extern "C" j2d_status j2d5pt_run_states(j2d5pt_plan_t p, const void *in, void *s
   // AUTO keeps states with the one-step kernel, which writes every state anyway, but
   // for FP64 grids of 8 M cells and more whose weights have a window, which take
   // the stream passes.  Microseconds a state, one-step and stream: 4096^2, noise 132 and
-  // 97, smooth positive fields 132 and 87, fields of both signs, which no window
+  // 94, smooth positive fields 132 and 87, fields of both signs, which no window
   // takes, 171 and 179; 2304x1700, six states, 37 and 45, 37 and 28, 49 and 53; weights without
   // a window, 4096^2: 135 and 140, with a zero or negative one 156 and 169.
   DtbConfig c = resolve(p, steps, false);

@@ -502,8 +502,8 @@ __device__ __forceinline__ void stream_sweep(const StreamParams &p, const typena
 // ---- FP64 in windowed fixed point (window.cuh) -----------------------------------
 // The same pipeline with every row also in fixed point: rows y mod 4 in {0, 1} take
 // the exact sum, the others the chain with its first two operations, on the
-// integer pipes.  A sweep picks its window from the first rows it reads and
-// stops before the first row that depends on an interior value outside it; the
+// integer pipes.  A sweep picks its window from the first interior rows it reads
+// and stops before the first row that depends on an interior value outside it; the
 // caller takes the next rows through stream_sweep() and comes back.  Ring values
 // never change, so a sweep does not stop for them: a row beside a ring value
 // outside the window takes its affected cells through the general evaluation.
@@ -526,8 +526,7 @@ template <> struct WindowCoef<9> {
 // that its doubles are not needed again.
 constexpr int kBoxHead = 3;
 
-// Rows [y0, y1) of the unit; returns the first row not stored (y1: all are), or
-// -1 when the first rows hold a value no window takes.
+// Rows [y0, y1) of the unit; returns the first row not stored (y1: all are).
 template <int M, bool EDGE, bool KEEP, int SH>
 __device__ __forceinline__ int stream_sweep_window(const StreamParams &p, const typename WindowCoef<SH>::L &lk, long e0, int x0,
                                                    unsigned hold, bool live, bool st, int y0, int y1, float4 *ring) {
@@ -547,18 +546,32 @@ __device__ __forceinline__ int stream_sweep_window(const StreamParams &p, const 
   // columns of this lane outside the logical array hold a value of the window
   const bool oa = EDGE && (x0 < 0 || x0 > p.nx + 1), ob = EDGE && (x0 + 1 < 0 || x0 + 1 > p.nx + 1);
   if (EDGE) hold |= (oa ? 1u : 0u) | (ob ? 2u : 0u);
-  // window: its top one binade above the largest interior value of the first rows
-  stage_drain();
+  // window: its top one binade above the largest value of the first kProbe interior
+  // rows.  They are read here beside their copies (the first copied rows may lie above
+  // the grid: M = 4, the first unit of a band), and a value below the window ends the
+  // attempt before its pipeline is filled.
+  constexpr int kProbe = 4;
+  const int r0 = max(a, 1);
+  double2 v[kProbe];
+#pragma unroll
+  for (int j = 0; j < kProbe; ++j) {
+    const long e = (long)(r0 + j) * p.pitch + e0;
+    v[j] = live && r0 + j <= p.ny && stream_ok(e, 2, p) ? __ldcg(reinterpret_cast<const double2 *>(in + e))
+                                                        : make_double2(1.0, 1.0);
+  }
+  const bool ka = live && !(EDGE && (hold & 1u)), kb = live && !(EDGE && (hold & 2u));  // interior columns
   int top = 0, low = 0x7fffffff;  // high words: negative for negative values
 #pragma unroll
-  for (int j = 0; j < kAhead; ++j) {
-    const double2 v = *reinterpret_cast<const double2 *>(ring + 32 * j);
-    if (a + j < 1 || a + j > p.ny) continue;
-    if (!EDGE || !(hold & 1u)) top = max(top, __double2hiint(v.x)), low = min(low, __double2hiint(v.x));
-    if (!EDGE || !(hold & 2u)) top = max(top, __double2hiint(v.y)), low = min(low, __double2hiint(v.y));
+  for (int j = 0; j < kProbe; ++j) {
+    if (r0 + j > p.ny) continue;
+    if (ka) top = max(top, __double2hiint(v[j].x)), low = min(low, __double2hiint(v[j].x));
+    if (kb) top = max(top, __double2hiint(v[j].y)), low = min(low, __double2hiint(v[j].y));
   }
   Window q;
-  if (!window_set(q, w, __reduce_max_sync(0xffffffffu, top) >> 20) || __any_sync(0xffffffffu, low < 0x100000)) return -1;
+  if (!window_set(q, w, __reduce_max_sync(0xffffffffu, top) >> 20) || __any_sync(0xffffffffu, low < (int)q.cref)) {
+    stage_drain();
+    return y0;
+  }
   const double dummy = window_dummy(q);
   RowX A[M], B[M];
   {
@@ -729,26 +742,24 @@ __device__ __forceinline__ int stream_sweep_window(const StreamParams &p, const 
 __device__ __forceinline__ const Links<double> &chain_of(const WeightsD &k) { return k.l; }
 __device__ __forceinline__ const Box9<double> &chain_of(const WeightsD9 &k) { return k.b; }
 
-// A unit in windowed fixed point where its values allow it; elsewhere stretches
-// of rows by the general sweep: eight rows, four times as many while the window
-// keeps failing soon after, and all of them where a value is not positive.
+// A unit in windowed fixed point; from the first row that depends on a value outside
+// the window, or at once when its first rows hold one, kWindowRetry rows by the
+// general sweep before the next attempt.  Units are seldom taller, so most try one
+// window a pass: a value that fits none has others near it, and each further attempt
+// costs its probe and two pipelines' filling (noise, three attempts a unit and one:
+// FP64 8192^2 x 4 1792 -> 1440 us, where the kernel without windows took 1620; box
+// 2048x1536 x 6 416 -> 320 us, 397 without).
+constexpr int kWindowRetry = 256;
 template <int M, bool EDGE, bool KEEP, int SH>
 __device__ __forceinline__ void stream_unit_window(const StreamParams &p, const typename RowOf<double, SH>::W &k, long e0, int x0,
                                                    unsigned hold, bool live, bool st, int y0, int y1, float4 *ring) {
-  const uint32_t lim = WindowCoef<SH>::window(p).lim;
-  int stretch = lim ? 8 : y1;
+  const bool window = WindowCoef<SH>::window(p).lim != 0;  // the weights have one
   while (y0 < y1) {
-    if (lim) {
-      const int y = stream_sweep_window<M, EDGE, KEEP, SH>(p, chain_of(k), e0, x0, hold, live, st, y0, y1, ring);
-      if (y < 0) stretch = y1;
-      else if (y - y0 >= 16) stretch = 8;
-      y0 = max(y, y0);
-    }
+    if (window) y0 = stream_sweep_window<M, EDGE, KEEP, SH>(p, chain_of(k), e0, x0, hold, live, st, y0, y1, ring);
     if (y0 < y1) {
-      const int ye = y0 + min(stretch, y1 - y0);
+      const int ye = window ? min(y0 + kWindowRetry, y1) : y1;
       stream_sweep<double, M, EDGE, true, KEEP, SH>(p, k, e0, x0, hold, live, st, y0, ye, ring);
       y0 = ye;
-      stretch = min(4 * stretch, 1 << 20);
     }
   }
 }
