@@ -33,10 +33,10 @@
 // same values in windowed fixed point where a unit's values allow it (window.cuh).
 // So the results are bit-identical to every other kernel of the library.
 //
-// One launch per pass (a pass waits for the one before it; a run of
-// S steps is ceil(S / M) passes, the first one taking the remainder), with
-// several waves of (band, run) units so that the block scheduler balances the
-// SMs.  Per cell update HBM carries 2 * sizeof(T) * (1 + overlap) / M bytes.
+// One launch per pass (a pass waits for the one before it; a run of S steps is
+// ceil(S / M) passes, the first one taking the remainder, which at two FP64 steps a
+// pass the one-step kernel takes), with several waves of (band, run) units so that
+// the block scheduler balances the SMs.  Per cell update HBM carries 2 * sizeof(T) * (1 + overlap) / M bytes.
 // The same pipeline serves the 3x3 box (j2d9pt) and, for state-keeping runs,
 // stores every step's rows instead of the last step's only.
 #include <algorithm>
@@ -954,9 +954,13 @@ StreamGeom stream_geometry_warps(j2d_dtype dt, int nx, int ny, int depth, long w
 
 // A pass of m <= q.depth steps, in -> out (distinct buffers whose rings
 // agree); with keep set, step t's state goes to keep + (t - 1) * keep_stride
-// elements instead (out unused).
+// elements instead (out unused).  The one step that a run of an odd number of steps
+// has over at two steps a pass is the one-step kernel's: a pass for it takes as long as
+// for two (4096^2 x 7, noise 810 -> 645 us, both signs 1433 -> 1248; box 1481 -> 1094 and
+// 2712 -> 2329; 100^2 x 7 box 125 -> 96).
 cudaError_t launch_stream_pass(j2d_dtype dt, const void *in, void *out, const GridDesc &g, const StreamGeom &q, int m,
                                int ipath, int *status, cudaStream_t s, void *keep, long keep_stride) {
+  if (dt == J2D_F64 && q.depth == 2 && m == 1) return launch_onestep(dt, false, in, keep ? keep : out, g, ipath, s);
   StreamParams p;
   p.in = in;
   p.out = out;
