@@ -236,12 +236,15 @@ __device__ __forceinline__ RowF9 row_step9(const WeightsF9 &k, const RowF9 &ym, 
   rb.y = __fmaf_rn(k.w[8].x, yp.R, rb.y);
   return {ra, rb, 0.f, 0.f};
 }
+// SKIP (windowed kernels, whose general sweep is for fields of both signs first of all):
+// the integer path wants nine positive normal values, which few of a row's 64 cells then
+// have, and a row without any skips the attempt (300 instructions a cell).  The test
+// also takes the two cells one after the other: deeper pipelines lose by it (k = 4,
+// 9000x8000 x 4 of both signs 7617 -> 9903 us).
+template <bool SKIP>
 __device__ __forceinline__ RowD9 row_step9(const WeightsD9 &k, const RowD9 &ym, const RowD9 &c, const RowD9 &yp,
                                            bool ea, bool eb) {
-  // the integer path wants nine positive normal values: in a field of both signs
-  // few of a row's 64 cells have them, and a row without any skips the attempt
-  // (300 instructions a cell)
-  if (ea || eb) {
+  if (SKIP && (ea || eb)) {
     const int lo = min(min(__double2hiint(ym.a), __double2hiint(ym.b)),
                        min(min(__double2hiint(c.a), __double2hiint(c.b)), min(__double2hiint(yp.a), __double2hiint(yp.b))));
     const int la = min(lo, min(__double2hiint(ym.L), min(__double2hiint(c.L), __double2hiint(yp.L))));
@@ -265,21 +268,25 @@ __device__ __forceinline__ void row_nbrs(RowD &) {}
 // ea, eb: the lane's first / second cell takes the integer path (FP64; known
 // at compile time where the trip's row phases are: the column parities of a
 // lane's two cells are fixed, its first column being odd).
+template <bool SKIP>
 __device__ __forceinline__ RowF step_any(const WeightsF &k, const RowF &ym, const RowF &c, const RowF &yp, bool,
                                          bool) {
   return row_step(k, ym, c, yp);
 }
+template <bool SKIP>
 __device__ __forceinline__ RowD step_any(const WeightsD &k, const RowD &ym, const RowD &c, const RowD &yp, bool ea,
                                          bool eb) {
   return row_step(k, ym, c, yp, ea, eb);
 }
+template <bool SKIP>
 __device__ __forceinline__ RowF9 step_any(const WeightsF9 &k, const RowF9 &ym, const RowF9 &c, const RowF9 &yp, bool,
                                           bool) {
   return row_step9(k, ym, c, yp);
 }
+template <bool SKIP>
 __device__ __forceinline__ RowD9 step_any(const WeightsD9 &k, const RowD9 &ym, const RowD9 &c, const RowD9 &yp,
                                           bool ea, bool eb) {
-  return row_step9(k, ym, c, yp, ea, eb);
+  return row_step9<SKIP>(k, ym, c, yp, ea, eb);
 }
 
 // In the checked build, is [e, e + V) inside the buffer of nelem elements?
@@ -289,6 +296,10 @@ __device__ __forceinline__ bool stream_ok(long e, int V, const StreamParams &p) 
   if (!ok) set_error(p.status, DEV_BOUNDS);
   return ok;
 }
+
+// Kernels whose units run in windowed fixed point.
+template <typename T, int M, bool IP, bool KEEP, int SH>
+constexpr bool kWindowed = std::is_same<T, double>::value && M <= (SH == 5 ? 4 : 2) && IP;
 
 // The pipeline of one warp: for each step t = 0..M-1 the two most recent rows
 // of step t (A: the older, B: the newer).
@@ -329,7 +340,7 @@ template <typename T, int M, bool EDGE, bool IP, bool KEEP, int SH> struct Pipe 
     for (int t = 1; t <= M; ++t) {
       const int r = i - t;  // the row step t evaluates
       const int yy = ph >= 0 ? ph - t + 4 * M : r;  // the row, or a row of the same phase mod 4
-      R n = step_any(k, A[t - 1], B[t - 1], cur, IP && exact_cell(1, yy, true), IP && exact_cell(0, yy, true));
+      R n = step_any<kWindowed<T, M, IP, KEEP, SH>>(k, A[t - 1], B[t - 1], cur, IP && exact_cell(1, yy, true), IP && exact_cell(0, yy, true));
       if (EDGE) n = row_hold(n, B[t - 1], hold);
       if (CHK && (r == 0 || r == p.ny + 1 || t > p.meff)) n = B[t - 1];
       if (SH == 9 && t < M) row_nbrs(n);  // read with its neighbours by steps t + 1 (three times)
@@ -787,22 +798,18 @@ __device__ __forceinline__ void make_weights(const StreamParams &p, WeightsD *k)
   k->u = exact_weights(l);
 }
 
-// Kernels whose units run in windowed fixed point.
-template <typename T, int M, bool IP, bool KEEP, int SH>
-constexpr bool kWindowed = std::is_same<T, double>::value && M <= (SH == 5 ? 4 : 2) && IP;
-
 // Resident blocks per SM asked of the compiler (0: its own choice).  Windowed, M = 2:
 // five blocks of four warps (96 registers, some spilled in the rare branches)
 // measured faster than four or six (FP64 16384^2: 259, 252 and 255 GCells/s); box:
 // four (144 at 16384^2; three 137, five 144; without the window 92).
-// Deep FP32 pipelines and the FP64 box: the occupancy they have had without
-// steady-trip registers on top (FP32 k = 12, 16384^2: 4126 GCells/s at 12 warps,
-// 3872 at 10).
+// Deep FP32 pipelines: the warps they had without steady-trip registers on top
+// (k = 12, 16384^2: 4126 GCells/s at 12 warps, 3872 at 10; box k = 8, 9000x8000 x 48:
+// 1587 us at 11, 1650 with the compiler's own choice of 196 registers).
 template <typename T, int M, bool IP, bool KEEP, int SH> constexpr int stream_blocks() {
   if (kWindowed<T, M, IP, KEEP, SH>) return SH == 9 ? 4 : 7 - M;
   if (KEEP) return 0;
   if (std::is_same<T, float>::value && SH == 5) return M == 10 ? 13 : M == 12 ? 12 : 0;
-  if (std::is_same<T, float>::value) return M == 8 ? 12 : 0;
+  if (std::is_same<T, float>::value) return M == 8 ? 11 : 0;
   return 0;
 }
 
