@@ -316,11 +316,16 @@ j2d_status j2d5pt_arith_info(unsigned *exact_mask, int *exact_guard);
  * stored columns per band (32 vectors' worth minus 2G), bands
  * (ceil(nx / stored columns)), rows stored per run H, runs per band}: band b
  * stores columns [1 + b*(stored), ...) and run r rows [1 + r*H, ...), each
- * clipped to the grid (runs too few to fill the device are each shared by
- * several warps).  J2D_ERR_ARG for sizes < 1, an unknown dtype or shape,
+ * clipped to the grid; where the runs are too few to fill the device, several
+ * warps share a run (j2d5pt_stream_units).  J2D_ERR_ARG for sizes < 1, an unknown dtype or shape,
  * a depth with no stream kernel, resident_warps < 1 or a NULL out. */
 j2d_status j2d5pt_stream_geometry(int nx, int ny, j2d_dtype dtype, int shape, int depth, long resident_warps,
                                   long out[6]);
+
+/* What the warps of that geometry store, as a pass launches them: out[0..1] = {rows
+ * per warp, warps per band}.  Warp u of band b stores rows [1 + u*rows, ...) of the band's
+ * columns, clipped to the grid; H is a multiple of the rows.  Errors as above. */
+j2d_status j2d5pt_stream_units(int nx, int ny, j2d_dtype dtype, int shape, int depth, long resident_warps, long out[2]);
 
 /* Number of CUDA kernels this library has launched in this process so far
  * (all threads, all plans); a diagnostic for launch accounting. */

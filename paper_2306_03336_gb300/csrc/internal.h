@@ -82,7 +82,8 @@ struct StreamGeom {
   int bands = 0;  // column bands
   int H = 0;      // rows stored per run
   int runs = 0;   // runs per band
-  int hu = 0;     // rows stored per warp: H, or a part of a run where the runs are too few to fill the device
+  int hu = 0;     // rows stored per warp: H, or a part of a run (H is a multiple of it) where the runs are too few to fill the device
+  int units = 0;  // warps per band: ceil(ny / hu)
 };
 int stream_max_depth(j2d_dtype dt);
 bool stream_depth_ok(j2d_dtype dt, int m, int shape = 5);  // a kernel of m steps per pass exists

@@ -944,8 +944,7 @@ StreamGeom stream_geometry_warps(j2d_dtype dt, int nx, int ny, int depth, long w
     // too few units of that height for one wave: the warps share the runs
     q.hu = (int)std::min<long>(q.H, std::max<long>(hu, 8));
   } else {
-    const int waves = dt == J2D_F64 ? 8 : 3;
-    int runs = (int)std::max<long>(1, waves * warps / q.bands);
+    int runs = (int)std::max<long>(1, 3 * warps / q.bands);
     runs = std::min(runs, std::max(1, ny / hmin));
     q.H = (ny + runs - 1) / runs;
     // smaller grids: one wave of shorter units, at least 3.5M rows (FP32 2048x1536,
@@ -955,7 +954,9 @@ StreamGeom stream_geometry_warps(j2d_dtype dt, int nx, int ny, int depth, long w
     const long r1 = std::max<long>(1, warps / q.bands);
     q.hu = (int)std::min<long>(q.H, std::max<long>((ny + r1 - 1) / r1, 7 * q.depth / 2));
   }
+  q.H = (q.H + q.hu - 1) / q.hu * q.hu;  // a run is a whole number of its warps' units
   q.runs = (ny + q.H - 1) / q.H;
+  q.units = (ny + q.hu - 1) / q.hu;
   return q;
 }
 
@@ -979,7 +980,7 @@ cudaError_t launch_stream_pass(j2d_dtype dt, const void *in, void *out, const Gr
   p.vw = q.vw;
   p.bands = q.bands;
   p.H = q.hu;
-  p.runs = (g.ny + q.hu - 1) / q.hu;
+  p.runs = q.units;
   p.meff = m;
   p.keep = keep;
   p.keep_stride = keep_stride;

@@ -90,6 +90,7 @@ def _open(path):
         "j2d5pt_measure_smem_bandwidth": [ctypes.POINTER(D)],
         "j2d5pt_arith_info": [ctypes.POINTER(ctypes.c_uint), ctypes.POINTER(I)],
         "j2d5pt_stream_geometry": [I, I, I, I, I, L, ctypes.POINTER(L)],
+        "j2d5pt_stream_units": [I, I, I, I, I, L, ctypes.POINTER(L)],
     }
     for name, args in sig.items():
         f = getattr(lib, name)
@@ -292,6 +293,13 @@ def j2d5pt_stream_geometry(nx, ny, dtype, depth, resident_warps, shape=5):
     _check(load().j2d5pt_stream_geometry(int(nx), int(ny), _DT[dtype], int(shape), int(depth), int(resident_warps),
                                          out))
     return dict(zip(("depth", "G", "vw", "bands", "H", "runs"), (int(v) for v in out)))
+
+
+def j2d5pt_stream_units(nx, ny, dtype, depth, resident_warps, shape=5):
+    """(rows stored per warp, warps per band) of that geometry, as a pass launches them."""
+    out = (ctypes.c_long * 2)()
+    _check(load().j2d5pt_stream_units(int(nx), int(ny), _DT[dtype], int(shape), int(depth), int(resident_warps), out))
+    return int(out[0]), int(out[1])
 
 
 _DT = {"f64": J2D_F64, "f32": J2D_F32, np.float64: J2D_F64, np.float32: J2D_F32}
