@@ -718,7 +718,12 @@ extern "C" j2d_status j2d5pt_sync_status(j2d5pt_plan_t p) {
 // takes under 5 ms (best of two or three runs after a warm-up run); the
 // fastest per step is kept in the plan.  With J2D_TUNE_CACHE set, results are
 // read from / appended to that file, keyed by device, SM count, dtype, grid
-// sizes and the step-count bucket.
+// sizes, what the integer path can do with a single grid's weights (the speed of the
+// FP64 stream passes hangs on it), the step-count bucket and kTuneRevision.
+
+// Raised when kernels change enough that choices tuned with the old ones are stale.
+constexpr int kTuneRevision = 2;
+
 static std::string tune_key(j2d5pt_plan_t p, long steps) {
   cudaDeviceProp prop;
   cudaGetDeviceProperties(&prop, p->device);
@@ -730,7 +735,8 @@ static std::string tune_key(j2d5pt_plan_t p, long steps) {
     h = (h ^ (unsigned long long)g.ny) * 1099511628211ull;
   }
   k += "|" + std::to_string(p->grids.size()) + "|" + std::to_string(h) + "|ip" + std::to_string(int_path_of(p)) +
-       "|sw" + std::to_string(p->opt_sweep_steps) + "|s" + std::to_string(p->grids[0].shape);
+       "|sw" + std::to_string(p->opt_sweep_steps) + "|s" + std::to_string(p->grids[0].shape) + "|w" +
+       std::to_string(p->grids.size() == 1 ? (int)weight_class(p) : 0) + "|r" + std::to_string(kTuneRevision);
   long b = 1;
   while (b < steps) b <<= 1;
   k += "|" + std::to_string(b);
