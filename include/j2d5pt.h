@@ -84,7 +84,7 @@ typedef enum {
                             grids only (adjoint runs and batches take TILES).  AUTO takes it for
                             FP32 grids and, in runs of six steps or more, for FP64 grids
                             too large for the chip (unless their weights are all positive
-                            and spread over more than about 100 times) and FP64 box grids
+                            and spread over about 100 to 2000 times) and FP64 box grids
                             whose weights lie within about 32 times of each other (FP64
                             grids of 8192^2 cells or more: from four steps on). */
 } j2d_algo;

@@ -2,6 +2,7 @@
 // dispatch to the one-step and temporally blocked kernels, host end-to-end
 // runs, status reporting.
 #include <cfloat>
+#include <climits>
 #include <cmath>
 #include <cstdint>
 #include <cstdarg>
@@ -290,8 +291,15 @@ static WeightClass weight_class(j2d5pt_plan_t p) {
   const GridDesc &g = p->grids[0];
   const int n = g.shape;  // five or nine weights
   if (!int_path_of(p)) return WEIGHTS_CHAIN;
-  for (int i = 0; i < n; ++i)
-    if (!(g.w[i] >= DBL_MIN)) return WEIGHTS_CHAIN;  // negative, zero or subnormal: every cell takes the chain
+  int lo = INT_MAX, hi = INT_MIN;
+  for (int i = 0; i < n; ++i) {
+    if (!(g.w[i] >= DBL_MIN)) return WEIGHTS_CHAIN;  // negative, zero or subnormal
+    lo = std::min(lo, std::ilogb(g.w[i]));
+    hi = std::max(hi, std::ilogb(g.w[i]));
+  }
+  // weights as far apart as the guard: even values of one size, as cells' are after a
+  // few steps, leave some (further apart: all) cells to the chain
+  if (hi - lo >= kExactGuard) return WEIGHTS_CHAIN;
   const uint32_t lim = n == 9 ? window_weights(box_chain<double>(g.w).w).lim
                               : window_weights({g.w[0], g.w[1], g.w[2], g.w[3], g.w[4]}).lim;
   return lim ? WEIGHTS_WINDOWED : WEIGHTS_POSITIVE;

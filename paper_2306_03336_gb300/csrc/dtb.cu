@@ -1902,11 +1902,11 @@ DtbConfig dtb_choose(j2d_dtype dt, const std::vector<GridDesc> &grids, int sms, 
     // 4254 GCells/s against 1950 for the best shared-memory schedule; the box
     // 2578 against 1418) and five-point FP64 (16384^2: 259 against 162 for the
     // tiles; 4096^2: 193 against 145; 2304x1700: 146 against 97; fields of both
-    // signs, which no window takes, 4096^2: 91 against 86; every cell a chain, as with
-    // a zero or negative weight or without the integer path: 100 against 87), and
-    // for large FP64 box grids.  Positive weights without a window stay with the
-    // tiles below 8192^2 (spread 2^10, 3001x4099: 121 and 115 GCells/s, tiles and
-    // stream, 4096^2: 140 and 126)
+    // signs, which no window takes, 4096^2: 91 against 86; cells that are chains, as with
+    // a zero or negative weight or without the integer path: 100 against 87), and for
+    // large FP64 box grids.  Positive weights without a window stay with the tiles below
+    // 8192^2 unless they are 2^11 apart or more (3001x4099, tiles and stream: 2^10 124
+    // and 117 GCells/s, 2^11 105 and 109, 2^12 77 and 91)
     else if (single && !rq.adjoint &&
              (dt == J2D_F32 || (grids[0].shape == 5 && rq.weights != WEIGHTS_POSITIVE && rq.steps >= 6 && depth_streams) ||
               (long)grids[0].nx * grids[0].ny >= (8192L << 13)))

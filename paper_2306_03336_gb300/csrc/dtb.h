@@ -10,9 +10,9 @@ struct j2d5pt_plan_s;
 
 namespace j2d {
 
-// What the FP64 integer path can do with a plan's weights: nothing (the path is off
-// or a weight is not positive normal, so every cell is an FMA chain), exact sums
-// cell by cell, or exact sums in windowed fixed point (window.cuh).
+// What the FP64 integer path can do with a plan's weights: next to nothing (the path is
+// off, a weight is not positive normal, or they are too far apart, so cells are FMA
+// chains), exact sums cell by cell, or exact sums in windowed fixed point (window.cuh).
 enum WeightClass { WEIGHTS_CHAIN, WEIGHTS_POSITIVE, WEIGHTS_WINDOWED };
 
 struct DtbRequest {

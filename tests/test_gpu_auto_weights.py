@@ -12,7 +12,9 @@ TINY = float(np.finfo(np.float64).tiny)
 FIVE = [  # weights, int_path, schedule of a grid too large for the chip
     ([0.5, 0.25, 0.04, 0.15, 0.06], 1, "stream"),
     ([0.55, 0.2, 0.0005, 0.1395, 0.11], 1, "tiles"),
-    ([0.55, 0.2, TINY, 0.13, 0.11], 1, "tiles"),
+    ([0.55, 0.2, 2.0 ** -11, 0.13, 0.11], 1, "tiles"),
+    ([0.55, 0.2, 0.99 * 2.0 ** -11, 0.13, 0.11], 1, "stream"),
+    ([0.55, 0.2, TINY, 0.13, 0.11], 1, "stream"),
     ([0.55, 0.2, TINY / 2, 0.13, 0.11], 1, "stream"),
     ([0.25, 0.25, 0.25, 0.0, 0.25], 1, "stream"),
     ([0.3, 0.3, -0.1, 0.25, 0.25], 1, "stream"),
