@@ -76,17 +76,18 @@ typedef enum {
   J2D_ALGO_STREAM = 6    /* temporal blocking in the register file: each warp sweeps a column
                             band (32 16-byte vectors wide, overlapped halo in x) down a run of
                             rows, advancing k steps per pass as a pipeline held in registers
-                            (step t of row i-t as row i arrives); one launch per pass, no shared
-                            memory.  k in {4, 6, 8, 10, 12} for FP32, {2, 3, 4, 6} for FP64
-                            (J2D_ERR_ARG otherwise; default 8, or 6 below 3200^2 cells unless
-                            the run has 7 or 8 steps, and 2);
-                            box plans: {4, 6, 8} for FP32, {2, 3, 4} for FP64 (default 6 and 2).  Forward runs of single
-                            grids only (adjoint runs and batches take TILES).  AUTO takes it for
-                            FP32 grids and, in runs of six steps or more, for FP64 grids
-                            too large for the chip (unless their weights are all positive
-                            and spread over about 100 to 2000 times) and FP64 box grids
-                            whose weights lie within about 32 times of each other (FP64
-                            grids of 8192^2 cells or more: from four steps on). */
+                            (step t of row i-t as row i arrives); one launch per pass, shared
+                            memory only for the rows on their way in.  k in {4, 6, 8, 10, 12}
+                            for FP32, {2, 3, 4, 6} for FP64 (J2D_ERR_ARG otherwise; default 8,
+                            or 6 below 3200^2 cells unless the run has 7 or 8 steps, and 2);
+                            box plans: {4, 6, 8} for FP32, {2, 3, 4} for FP64 (default 6, or 8
+                            for runs of 7 or 8 steps, and 2).  Forward runs of single grids
+                            only (adjoint runs and batches take TILES).  AUTO takes it from four
+                            steps on for FP32 grids and for FP64 grids too large for the chip
+                            (below 8192^2 cells not where the weights are all positive and
+                            spread over about 100 to 2000 times), and from six steps on for
+                            FP64 box grids whose weights lie within about 32 times of each
+                            other (from four at 8192^2 cells or more, whatever the weights). */
 } j2d_algo;
 
 /* Plan options (j2d5pt_set_option / j2d5pt_get_option). */
@@ -190,7 +191,7 @@ j2d_status j2d5pt_run_host(j2d5pt_plan_t plan, const void *h_in, void *h_out, lo
  * (ny+2) * pitch elements.  Bit-identical to `steps` chained calls of
  * j2d5pt_run(plan, ., ., 1, stream).  With J2D_ALGO_AUTO FP64
  * grids of 8 M cells or more whose weights have a window (see
- * J2D_ALGO_STREAM) take the stream passes from six states on, others the one-step
+ * J2D_ALGO_STREAM) take the stream passes from four states on, others the one-step
  * kernel, one launch per state (it writes every state anyway); a plan set to a
  * temporally blocked algorithm stores each state from its one persistent
  * launch (the skewed and two-step FP32 schedules run as single-step tiles

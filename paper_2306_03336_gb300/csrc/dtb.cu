@@ -1549,8 +1549,8 @@ __device__ Strip slot_strip(const int *rec, int SWc) {
 // to its buffer d (1 = workspace, 2 = output), gridDim.z blocks sharing it, and
 // the blocks together reset the barrier counter (the first 64 words of `scratch`) and
 // the step counters after it (nflags words, to -1).  In place of two memset
-// launches and one 256-thread block per ring (FP64 200x120 x 12 steps: 68 -> 62 us,
-// 512^2 x 16: 106 -> 102).
+// launches and one 256-thread block per ring (FP64 200x120 x 12 steps: 58.3 -> 54.0 us,
+// 512^2 x 16: 96.5 -> 90.3).
 constexpr int kSetupThreads = 1024;
 template <typename T>
 __global__ void __launch_bounds__(kSetupThreads) setup_kernel(const GridDev *grids, int copy_ws, int copy_out, int *scratch,
@@ -1891,29 +1891,31 @@ DtbConfig dtb_choose(j2d_dtype dt, const std::vector<GridDesc> &grids, int sms, 
     // size (2048x1536: 1.9 against 3.3 us a step, 1024^2: 1.8 against 2.7, 512^2: 1.4
     // against 2.0)
     // FP64 box grids whose weights fit the windowed fixed point: the stream schedule
-    // at every size (4096^2: 150 us a step against 231 for the skewed tiles,
-    // 2048x1536: 42 against 63, 512^2: 16 against 29; fields of both signs, which no
-    // window takes, 330 against 319, 90 against 86, 28 against 37).  Not for four or
-    // five steps: the first pass over noise takes the general sweep (1500^2, four
-    // steps: 277 us against 237; eight: 393 against 486)
+    // at every size (4096^2 x 64: 145 us a step against 229 for the skewed tiles,
+    // 2048x1536: 41 against 63, 512^2: 15 against 29; fields of both signs, which no
+    // window takes, 328 against 319, 78 against 86, 23 against 37; 6000x5000: 564 against
+    // 533).  Not for four or five steps, where those fields and noise, whose first pass
+    // fits no window, are level with the tiles (4096^2 x 4: 1270 us against 1251 and 857
+    // against 928; 512^2 x 4: 92 against 115 and 106 against 104)
     else if (grids[0].shape == 9 && rq.weights == WEIGHTS_WINDOWED && rq.steps >= 6 && depth_streams) algo = J2D_ALGO_STREAM;
     else if (fits && (dt == J2D_F64 || (single && (rq.adjoint || !depth_streams)))) algo = J2D_ALGO_RESIDENT;
-    // grids too large for the chip: the stream schedule for FP32 (16384^2:
-    // 4254 GCells/s against 1950 for the best shared-memory schedule; the box
-    // 2578 against 1418) and five-point FP64 (16384^2: 259 against 162 for the
-    // tiles; 4096^2: 193 against 145; 2304x1700: 146 against 97; fields of both
-    // signs, which no window takes, 4096^2: 91 against 86; cells that are chains, as with
-    // a zero or negative weight or without the integer path: 100 against 87), and for
-    // large FP64 box grids.  Positive weights without a window stay with the tiles below
-    // 8192^2 unless they are 2^11 apart or more (3001x4099, tiles and stream: 2^10 124
-    // and 117 GCells/s, 2^11 105 and 109, 2^12 77 and 91)
+    // grids too large for the chip: the stream schedule for FP32 (16384^2: 4660
+    // GCells/s against 1950 for the best shared-memory schedule; the box 2744 against
+    // 1418) and five-point FP64 (48 steps, stream and tiles, GCells/s: 8192^2 241 and 157,
+    // 4096^2 197 and 145, 2304x1700 151 and 98; fields of both signs, which no window
+    // takes, 101 and 91, 95 and 87, 77 and 61; cells that are chains, as with a zero or
+    // negative weight or without the integer path, 4096^2: 100 and 87; four steps of noise,
+    // whose first pass fits no window, 4096^2: 149 and 132, 2304x1700: 99 and 86), and
+    // for large FP64 box grids.  Positive weights without a window stay with the tiles
+    // below 8192^2 unless they are 2^11 apart or more (3001x4099, tiles and stream: 2^10
+    // 124 and 117 GCells/s, 2^11 105 and 109, 2^12 77 and 91)
     else if (single && !rq.adjoint &&
-             (dt == J2D_F32 || (grids[0].shape == 5 && rq.weights != WEIGHTS_POSITIVE && rq.steps >= 6 && depth_streams) ||
+             (dt == J2D_F32 || (grids[0].shape == 5 && rq.weights != WEIGHTS_POSITIVE && depth_streams) ||
               (long)grids[0].nx * grids[0].ny >= (8192L << 13)))
       algo = J2D_ALGO_STREAM;
-    // FP64 adjoint runs of larger grids: the one-step kernel (4096^2: 98 us a step
-    // against 134 for the tiles, 2304x1700: 28 against 49; fields of both signs 163
-    // against 198 and 46 against 66)
+    // FP64 adjoint runs of larger grids: the one-step kernel (4096^2: 99 us a step
+    // against 132 for the tiles, 2304x1700: 26 against 48; fields of both signs 164
+    // against 196 and 46 against 66)
     else if (single && rq.adjoint && dt == J2D_F64) algo = J2D_ALGO_ONESTEP;
     else algo = J2D_ALGO_TILES;
   }
