@@ -647,11 +647,12 @@ extern "C" j2d_status j2d5pt_run_states(j2d5pt_plan_t p, const void *in, void *s
   cudaError_t e;
   if ((e = launch_ring_copy(p->dtype, in, states, g, s, steps, se)) != cudaSuccess) return cuda_fail(e, "run_states: rings");
   // AUTO keeps states with the one-step kernel, which writes every state anyway, but
-  // for FP64 grids of 8 M cells and more whose weights have a window, which take
-  // the stream passes.  Microseconds a state, one-step and stream: 4096^2, noise 132 and
-  // 94, smooth positive fields 132 and 87, fields of both signs, which no window
-  // takes, 171 and 179; 2304x1700, six states, 37 and 45, 37 and 28, 49 and 53; weights without
-  // a window, 4096^2: 135 and 140, with a zero or negative one 156 and 169.
+  // for FP64 grids of 8 M cells and more whose weights have a window, which take the
+  // stream passes.  Microseconds a state, one-step and stream, 24 states of noise,
+  // of a smooth positive field and of one of both signs, which no window takes: 4096^2 132
+  // and 92, 132 and 87, 172 and 178; 3001x2999 73 and 55, 73 and 51, 98 and 104;
+  // 2304x1700 36 and 29, 36 and 26, 48 and 52 (six states of noise: 37 and 36).  Weights
+  // without a window, 4096^2: 135 and 140, with a zero or negative one 156 and 169.
   DtbConfig c = resolve(p, steps, false);
   if (p->opt_algo == J2D_ALGO_AUTO &&
       !(c.algo == J2D_ALGO_STREAM && p->dtype == J2D_F64 && weight_class(p) == WEIGHTS_WINDOWED &&

@@ -241,6 +241,7 @@ __global__ void __launch_bounds__(256, WG || (ADJ && sizeof(T) == 4) ? 2 : 0) on
       done = adjoint_item_window<ROWS>(t, in, out, pitch, pc0, xw0, y0, nx, ny, wl, win);
     if (!WG && done) continue;
   }
+  // computed for items done already too: behind a test the fused pass spills 88 bytes
   Links<T> cw[V];  // links of this thread's columns on rows away from the ring
   ExactW cu[V];    // the same links unpacked for the integer path (FP64)
 #pragma unroll

@@ -13,12 +13,13 @@
 // overflow (b0s = 8 * b0 gives a1 * b0 the weight of a0 * b1):
 //   S0 = sum a0 b0 < 5 * 2^61, S1 = S0 >> 29 + sum (a0 b1 + a1 b0s),
 //   S2 = S1 >> 32 + sum a1 b1.
-// S1 is bounded by the plan's own weights (window_weights()): it stays below 2^64
-// for every exponent spread h up to 5 and, for weights of a comparable sum, 7.
-// k = 7 for h <= 4, else 3, so k + h <= 11 = kExactGuard, so every windowed cell satisfies the integer path's contract and
-// its correctly rounded sum is the result stencil_exact() gives: bit for bit the
-// same, at about 50 instructions per cell instead of 166 (350 against 150
-// Gcells/s measured alone at 1.99 GHz, register operands).
+// S1 is bounded by the plan's own weights (window_weights()): of random normalised
+// weights it stays below 2^64 for every set of an exponent spread h up to 6 and one in five
+// of h = 7 (nine terms, below: up to 4, and one set in four of h = 5).  k = 7 for
+// h <= 4, else 3, so k + h <= 11 = kExactGuard, so every windowed cell satisfies the
+// integer path's contract and its correctly rounded sum is the result stencil_exact()
+// gives: bit for bit the same, at about 50 instructions per cell instead of 166 (350
+// against 150 Gcells/s measured alone at 1.99 GHz, register operands).
 //
 // The FMA chain's first product and its first FMA are evaluated the same way
 // (window_mul, window_mul_fma: each rounded once, as the FP64 pipe rounds them),
@@ -36,7 +37,8 @@
 namespace j2d {
 
 // The nine-term box cell works the same way with W split at bit 28 (J below), so
-// that nine products still fit the columns.
+// that nine products still fit the columns.  A quarter of random nine-weight sets have
+// no window (most for S1), four in a hundred five-weight ones.
 
 // Weights in fixed point, in the cell's term order: xm, xp, ym, c, yp (NT = 5), or
 // the box's chain order (NT = 9).
