@@ -557,26 +557,31 @@ __device__ __forceinline__ int stream_sweep_window(const StreamParams &p, const 
   // columns of this lane outside the logical array hold a value of the window
   const bool oa = EDGE && (x0 < 0 || x0 > p.nx + 1), ob = EDGE && (x0 + 1 < 0 || x0 + 1 > p.nx + 1);
   if (EDGE) hold |= (oa ? 1u : 0u) | (ob ? 2u : 0u);
-  // window: its top one binade above the largest value of the first kProbe interior
-  // rows.  They are read here beside their copies (the first copied rows may lie above
-  // the grid: M = 4, the first unit of a band), and a value below the window ends the
-  // attempt before its pipeline is filled.
-  constexpr int kProbe = 4;
+  // window: its top one binade above the largest value of the rows probed, the first
+  // four interior ones and four spread over the unit, read here beside the copies
+  // (whose first rows may lie above the grid: M = 4, the first unit of a band).  A value
+  // of theirs below the window ends the attempt before its pipeline is filled.  With
+  // the first rows alone, fields that rise down a unit ran out of its window, and steep ones
+  // out of every other (64 steps of the box, 4096^2: a field growing by 2% a cell 24.0
+  // -> 14.8 ms, where the skewed tiles take 15.0; 1 + sin / 2 with weights that leave four
+  // binades 13.3 -> 9.5).
   const int r0 = max(a, 1);
-  double2 v[kProbe];
-#pragma unroll
-  for (int j = 0; j < kProbe; ++j) {
-    const long e = (long)(r0 + j) * p.pitch + e0;
-    v[j] = live && r0 + j <= p.ny && stream_ok(e, 2, p) ? __ldcg(reinterpret_cast<const double2 *>(in + e))
-                                                        : make_double2(1.0, 1.0);
-  }
   const bool ka = live && !(EDGE && (hold & 1u)), kb = live && !(EDGE && (hold & 2u));  // interior columns
   int top = 0, low = 0x7fffffff;  // high words: negative for negative values
 #pragma unroll
-  for (int j = 0; j < kProbe; ++j) {
-    if (r0 + j > p.ny) continue;
-    if (ka) top = max(top, __double2hiint(v[j].x)), low = min(low, __double2hiint(v[j].x));
-    if (kb) top = max(top, __double2hiint(v[j].y)), low = min(low, __double2hiint(v[j].y));
+  for (int part = 0; part < 2; ++part) {
+    double2 v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int r = min(part == 0 ? r0 + j : y0 + (j + 1) * (y1 - 1 - y0) / 4, p.ny);
+      const long e = (long)r * p.pitch + e0;
+      v[j] = live && stream_ok(e, 2, p) ? __ldcg(reinterpret_cast<const double2 *>(in + e)) : make_double2(1.0, 1.0);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (ka) top = max(top, __double2hiint(v[j].x)), low = min(low, __double2hiint(v[j].x));
+      if (kb) top = max(top, __double2hiint(v[j].y)), low = min(low, __double2hiint(v[j].y));
+    }
   }
   Window q;
   if (!window_set(q, w, __reduce_max_sync(0xffffffffu, top) >> 20) || __any_sync(0xffffffffu, low < (int)q.cref)) {

@@ -78,3 +78,23 @@ def test_second_attempt_in_a_tall_unit():
     plan.sync()
     assert torch.equal(plan.view(got), plan.view(ref))
     plan.close()
+
+
+@pytest.mark.parametrize("name", ["rise", "fall", "steep", "diagonal", "crossing"])
+@pytest.mark.parametrize("nx,ny", [(130, 9), (187, 301), (61, 1203)])
+def test_sloping_fields(name, nx, ny):
+    """Fields whose exponents drift down a unit: into its window and out of it, with weights
+    that leave eight binades and four."""
+    y, x = np.arange(ny + 2)[:, None], np.arange(nx + 2)[None, :]
+    u = {"rise": 2.0 ** (y / 30 + 0 * x), "fall": 2.0 ** (-y / 30 + 0 * x), "steep": 2.0 ** (y / 3 % 200 + 0 * x),
+         "diagonal": 2.0 ** ((x + y) / 37 % 60), "crossing": 1 + 0.5 * np.sin(y / 20) * np.cos(x / 30)}[name]
+    u = u * (1 + 2.0 ** -20 * np.random.default_rng(9).random(u.shape))
+    narrow5 = np.array([0.55, 0.2, 0.0085, 0.13, 0.1115])
+    narrow9 = np.array([0.25, 0.0085, 0.09, 0.12, 0.15, 0.11, 0.07, 0.1315, 0.07])
+    for make, depths in ((lambda: j2d5pt.Plan(nx, ny, "f64", W5), (2, 3, 4)),
+                         (lambda: j2d5pt.Plan(nx, ny, "f64", narrow5), (2, 4)),
+                         (lambda: j2d5pt.Plan.box9(nx, ny, "f64", W9), (2,)),
+                         (lambda: j2d5pt.Plan.box9(nx, ny, "f64", narrow9), (2,))):
+        ref = run(make, u, 8, "onestep", 0)
+        for depth in depths:
+            assert np.array_equal(run(make, u, 8, "stream", depth), ref), depth
